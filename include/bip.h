@@ -62,7 +62,10 @@ typedef enum {
 } bip_status;
 
 typedef enum {
-    BIP_PREC_FP32 = 0,         /* FP32 SIMT complex GEMMs                     */
+    BIP_PREC_FP32 = 0,         /* FP32 throughout: complex64 operands, each
+                                  element taken to the tensor cores as three
+                                  BF16 terms (24 bits, six products), FP32
+                                  sums; an infinite element gives NaN        */
     BIP_PREC_SPLIT_BF16 = 1,   /* tcgen05, every contraction in BF16 hi+lo
                                   (3 products per real product), FP32 acc.    */
     BIP_PREC_MIXED = 2,        /* tcgen05, coupling and Gram in BF16 (one
@@ -515,6 +518,19 @@ bip_status bip_build_s1_noalloc(bip_ctx* ctx, const float* V, const bip_atom* at
 bip_status bip_set_wait_limit(bip_ctx* ctx, int64_t ns);
 bip_status bip_debug_fail_alloc(int64_t k);
 bip_status bip_debug_allocs(int64_t* live, int64_t* made);
+
+/* The FP32 complex contraction under the FP32 precision and the reverse
+ * pass, by itself, for validation:
+ *   C[z][m][n] = sum_kb sum_k opA(A(z, m, kb, k) w[k]) opB(B(z, kb, k, n)),
+ * kb < blocks, k < K; op = conj with flag 1 (A) or 2 (B); flag 4: only the
+ * tiles that reach the diagonal or lie right of it (the rest of C is left as
+ * it is).  sA, sB: element strides of a row (m or n), of k, of the batch and
+ * of a block of k; of each operand's first two one is 1.  w (float32 [K],
+ * nullable): with blocks = 1 only.  A, B, C complex64 device, C [batch][M][N].
+ * BIP_ERR_INVALID_ARG for a null pointer, a size below 1 or such strides. */
+bip_status bip_debug_cgemm(bip_ctx* ctx, int32_t M, int32_t N, int32_t K, int32_t blocks, int32_t batch,
+                           const void* A, const int64_t* sA, const void* B, const int64_t* sB, int32_t flags,
+                           const float* w, void* C, void* stream);
 
 /* Text of the last error on this context ("" if none; static text if ctx
  * is NULL). */

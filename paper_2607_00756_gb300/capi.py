@@ -69,6 +69,7 @@ def _load():
         "bip_set_wait_limit": [VP, ctypes.c_int64],
         "bip_debug_fail_alloc": [ctypes.c_int64],
         "bip_debug_allocs": [P(ctypes.c_int64), P(ctypes.c_int64)],
+        "bip_debug_cgemm": [VP, I32, I32, I32, I32, I32, VP, P(ctypes.c_int64), VP, P(ctypes.c_int64), I32, VP, VP, VP],
         "bip_qeels_bins": [VP, I32, P(I32), P(I32)],
         "bip_coreloss_qeels": [VP, VP, P(D), I32, I32, VP, VP],
         "bip_copy_stash": [VP, I32, I32, VP, VP],
@@ -298,6 +299,16 @@ def bip_set_wait_limit(ctx, ns):
 
 def bip_debug_fail_alloc(k):
     _check("bip_debug_fail_alloc", None, _lib.bip_debug_fail_alloc(int(k)))
+
+
+def bip_debug_cgemm(ctx, M, N, K, blocks, batch, A, sA, B, sB, flags, w, C, stream=None):
+    """The FP32 complex contraction by itself; A, B: complex64 CUDA tensors
+    (their storage, addressed by the strides), C contiguous [batch, M, N]."""
+    arr = ctypes.c_int64 * 4
+    _check("bip_debug_cgemm", ctx,
+           _lib.bip_debug_cgemm(ctx, M, N, K, blocks, batch, ctypes.c_void_p(A.data_ptr()), arr(*sA),
+                                ctypes.c_void_p(B.data_ptr()), arr(*sB), flags, _dev(w), _dev(C), _stream(stream)))
+    return C
 
 
 def bip_debug_allocs():

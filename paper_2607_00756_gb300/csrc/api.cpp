@@ -81,6 +81,7 @@ struct bip_ctx {
     int occ_n = 0;                      // sites they were given for (0: none)
     DevBuf g_s1, g_w, g_R, g_gmt, g_T, g_D, g_Dsum;   // gradient pass workspaces
     DevBuf g_s1bar, g_s2bar, g_ubar, g_dA, g_dt1, g_dt2, g_adj, g_ckpt, g_seg, g_gvp;
+    DevBuf gpart;                       // parts of a split k range (cgemm_f32.cu)
     DevBuf g_tA, g_tB, g_sA2, g_sB2;    // split-BF16 operands of the reverse-pass contractions
     DevBuf cubeA, cubeB, cube_work, cube_mask;   // the cube on tcgen05
     DevBuf cube_grp, cube_wmap, mpart;  // cube-mode work groups; map modes' item map and column sums
@@ -809,7 +810,7 @@ bip_status bip_destroy(bip_ctx* c) {
                      &c->ray, &c->rax, &c->g_tA, &c->g_tB, &c->g_sA2, &c->g_sB2, &c->cubeA, &c->cubeB,
                      &c->cube_work, &c->cube_mask, &c->s1t, &c->psi, &c->ybuf, &c->cube_grp, &c->cube_wmap, &c->mpart,
                      &c->hcube, &c->shcube, &c->cstash, &c->ccols, &c->xopA, &c->xopB, &c->xm32, &c->tcache,
-                     &c->cr_ay, &c->cr_ax, &c->cr_cy, &c->cr_cx, &c->cr_T, &c->nf_count, &c->tw512, &c->cols2};
+                     &c->cr_ay, &c->cr_ax, &c->cr_cy, &c->cr_cx, &c->cr_T, &c->nf_count, &c->tw512, &c->cols2, &c->gpart};
     for (DevBuf* b : all) release(*b);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -944,11 +945,54 @@ void release_map_workspaces(bip_ctx* c, cudaStream_t s) {
         cudaGetLastError();
         return;
     }
-    for (DevBuf* b : {&c->opA32, &c->opB32, &c->mt32, &c->q32, &c->opA16, &c->opB16, &c->mt16, &c->q16,
+    for (DevBuf* b : {&c->opA32, &c->opB32, &c->mt32, &c->q32, &c->gpart, &c->opA16, &c->opB16, &c->mt16, &c->q16,
                       &c->op8A, &c->op8B, &c->gdiff, &c->cubeA, &c->cubeB, &c->cube_mask, &c->mpart,
                       &c->s1t, &c->psi, &c->ybuf, &c->xtc, &c->f8pmax, &c->f8inv0, &c->f8inv1, &c->f8sA,
                       &c->f8sB})
         release(*b);
+}
+
+// One FP32 contraction of cgemm_f32.cu: its plan, the workspace of a split k
+// range, the launch.
+cudaError_t cgemm(bip_ctx* c, CGemmF32 p, cudaStream_t s) {
+    size_t part = 0;
+    cudaError_t e = bip_cgemm_plan(p, &part);
+    if (e != cudaSuccess) return e;
+    if (part > 0) {
+        e = ensure(c->gpart, part * sizeof(float2), false, s);
+        if (e != cudaSuccess) return e;
+    }
+    p.part = (float2*)c->gpart.p;
+    p.err = (int*)c->errflag.p;
+    p.wait_ns = c->wait_ns;
+    return bip_cgemm_f32(p, s);
+}
+
+// The coupling in FP32: M = A B^T of nb sites, A [Dp][K] the detector side
+// (rows d), B [n_rows][K] the aperture side (rows (ch, b)), written transposed
+// as Mt[b][ch Dp + d] for the Gram step (ep_B = Bpad).
+CGemmF32 coupling_f32(int n_det, int n_rows, int K, const void* A, int64_t sA, const void* B, int64_t sB, void* C,
+                      int64_t ldc, int64_t sC, int Bpad, int Dp, int nb) {
+    CGemmF32 p{};
+    p.M = n_det; p.N = n_rows; p.batch = nb;
+    p.A = CGemmOperand{(const float2*)A, K, 1, sA, K, 1, 0, 0, 0};
+    p.B = CGemmOperand{(const float2*)B, K, 1, sB, K, 1, 0, 0, 0};
+    p.C = (float2*)C; p.scn = ldc; p.scb = sC;
+    p.ep_B = Bpad; p.ep_Dp = Dp;
+    return p;
+}
+
+// The Gram matrix in FP32, Q = conj(Mt) Mt^T over K = (ch, d).  tri: only its
+// upper triangle (what the scan polynomial reads).
+CGemmF32 gram_f32(int Bpad, int64_t ldm, const void* Mt, int64_t sM, void* Q, int64_t sQ, bool tri, int nb) {
+    CGemmF32 p{};
+    p.M = Bpad; p.N = Bpad; p.batch = nb;
+    p.A = CGemmOperand{(const float2*)Mt, ldm, 1, sM, (int)ldm, 1, 0, 0, 0};
+    p.B = p.A;
+    p.conjA = 1;
+    p.C = (float2*)Q; p.scm = Bpad; p.scb = sQ;
+    p.tri = tri ? 1 : 0;
+    return p;
 }
 
 // Gather arguments of one side (1: S1 windows of the aperture beams,
@@ -1636,8 +1680,8 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
             CUDA_TRY(c, ensure(c->psi, SB * P128 * K * sizeof(float2), true, s));
             CUDA_TRY(c, ensure(c->ybuf, SB * 2 * P64r * nch * K * sizeof(uint16_t), true, s));
         }
-        CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     }
+    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     CUDA_TRY(c, ensure(c->q32, SB * perQ * sizeof(float2), true, s));
     // G(Delta) of every site when the raster evaluation runs once at the end,
     // else of one batch
@@ -2051,15 +2095,9 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
             TIMED(c, BIP_STAGE_GRAM, s, bip_tc_gemm(Gq, s));
         } else {
             // coupling M = S2^T diag(H) S1, stored transposed for the Gram step
-            CGemmArgs A{};
-            A.M = geo.n_det; A.N = (int)rowsB; A.K = K;
-            A.A = (const float2*)c->opA32.p; A.lda = K; A.strideA = (int64_t)perA;
-            A.Bm = (const float2*)c->opB32.p; A.ldb = K; A.strideB = (int64_t)perB;
-            A.batch = nb;
-            A.epi = 1;
-            A.C = (float2*)c->mt32.p; A.ldc = (int64_t)nch * Dpad; A.strideC = (int64_t)perMt;
-            A.ep_B = Bpad; A.ep_Dp = Dpad;
-            TIMED(c, BIP_STAGE_COUPLING, s, bip_cgemm_simt(A, s));
+            TIMED(c, BIP_STAGE_COUPLING, s,
+                  cgemm(c, coupling_f32(geo.n_det, (int)rowsB, K, c->opA32.p, (int64_t)perA, c->opB32.p, (int64_t)perB,
+                                        c->mt32.p, (int64_t)nch * Dpad, (int64_t)perMt, Bpad, Dpad, nb), s));
             if (sepq) {
                 CubeRasterArgs r = cra;
                 r.n_sites = nb;
@@ -2077,16 +2115,10 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
                 TIMED(c, BIP_STAGE_QUADFORM, s, bip_cube_accumulate(ca, s));
                 continue;
             }
-            // Gram Q = sum_n M^(n)H M^(n)
-            CGemmArgs Bq{};
-            Bq.M = Bpad; Bq.N = Bpad; Bq.K = nch * Dpad;
-            Bq.A = (const float2*)c->mt32.p; Bq.lda = (int64_t)nch * Dpad; Bq.strideA = (int64_t)perMt;
-            Bq.Bm = Bq.A; Bq.ldb = Bq.lda; Bq.strideB = Bq.strideA;
-            Bq.conjA = 1;
-            Bq.batch = nb;
-            Bq.epi = 0;
-            Bq.C = (float2*)c->q32.p; Bq.ldc = Bpad; Bq.strideC = (int64_t)perQ;
-            TIMED(c, BIP_STAGE_GRAM, s, bip_cgemm_simt(Bq, s));
+            // Gram Q = sum_n M^(n)H M^(n), upper triangle
+            TIMED(c, BIP_STAGE_GRAM, s,
+                  cgemm(c, gram_f32(Bpad, (int64_t)nch * Dpad, c->mt32.p, (int64_t)perMt, c->q32.p, (int64_t)perQ, true,
+                                    nb), s));
         }
         // I_tau(rho) = f_y f_x c^H Q c as a trigonometric polynomial over
         // beam-lattice differences, on the site's crop-window scan tiles
@@ -2131,7 +2163,7 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
         d.partial = partial;
         TIMED(c, BIP_STAGE_QUADFORM, s, bip_raster_eval(d, rargs, s));
     }
-    if (tc && !c->capture_safe) {
+    if (!c->capture_safe) {
         int flag = 0;
         CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(c, cudaStreamSynchronize(s));
@@ -2272,7 +2304,7 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
     CUDA_TRY(c, ensure(c->xopA, SB * perA * 8, true, s));
     CUDA_TRY(c, ensure(c->xopB, SB * perB * 8, true, s));
     CUDA_TRY(c, ensure(c->xm32, SB * perMt * sizeof(float2), true, s));
-    if (tc) CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
+    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
 
     // On a raster scan list the per-beam contraction separates over the
     // aperture beams' lattice (cube_raster.cu)
@@ -2498,15 +2530,9 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
                                       Bpad, s));
                 }
             } else {
-                CGemmArgs A{};
-                A.M = nd; A.N = (int)rowsB; A.K = K;
-                A.A = (const float2*)c->xopA.p; A.lda = K; A.strideA = (int64_t)perA;
-                A.Bm = (const float2*)c->xopB.p; A.ldb = K; A.strideB = (int64_t)perB;
-                A.batch = nb;
-                A.epi = 1;
-                A.C = (float2*)c->xm32.p; A.ldc = (int64_t)nch * Dpb; A.strideC = (int64_t)perMt;
-                A.ep_B = Bpad; A.ep_Dp = Dpb;
-                TIMED(c, BIP_STAGE_COUPLING, s, bip_cgemm_simt(A, s));
+                TIMED(c, BIP_STAGE_COUPLING, s,
+                      cgemm(c, coupling_f32(nd, (int)rowsB, K, c->xopA.p, (int64_t)perA, c->xopB.p, (int64_t)perB,
+                                            c->xm32.p, (int64_t)nch * Dpb, (int64_t)perMt, Bpad, Dpb, nb), s));
                 if (sep) {
                     CubeRasterArgs r = cra;
                     r.n_sites = nb;
@@ -2529,7 +2555,7 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
             }
         }
     }
-    if (tc && !c->capture_safe) {
+    if (!c->capture_safe) {
         int flag = 0;
         CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(c, cudaStreamSynchronize(s));
@@ -2633,6 +2659,32 @@ bip_status bip_debug_fail_alloc(int64_t k) {
 bip_status bip_debug_allocs(int64_t* live, int64_t* made) {
     if (live) *live = g_live.load();
     if (made) *made = g_made.load();
+    return BIP_OK;
+}
+
+bip_status bip_debug_cgemm(bip_ctx* c, int32_t M, int32_t N, int32_t K, int32_t blocks, int32_t batch, const void* A,
+                           const int64_t* sA, const void* B, const int64_t* sB, int32_t flags, const float* w, void* C,
+                           void* stream) {
+    if (!c || !A || !sA || !B || !sB || !C) return BIP_ERR_INVALID_ARG;
+    if (M < 1 || N < 1 || K < 1 || blocks < 1 || batch < 1 || (w && blocks != 1) || (sA[0] != 1 && sA[1] != 1) ||
+        (sB[0] != 1 && sB[1] != 1))
+        return fail(c, BIP_ERR_INVALID_ARG, "bad size or stride");
+    cudaStream_t s = (cudaStream_t)stream;
+    bip_status st = make_tables(c, s);
+    if (st != BIP_OK) return st;
+    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
+    CGemmF32 p{};
+    p.M = M; p.N = N; p.batch = batch;
+    p.A = CGemmOperand{(const float2*)A, sA[0], sA[1], sA[2], K, blocks, sA[3], 0, 0};
+    p.B = CGemmOperand{(const float2*)B, sB[0], sB[1], sB[2], K, blocks, sB[3], 0, 0};
+    p.conjA = flags & 1; p.conjB = flags >> 1 & 1; p.tri = flags >> 2 & 1;
+    p.dk = w;
+    p.C = (float2*)C; p.scm = N; p.scb = (int64_t)M * N;
+    CUDA_TRY(c, cgemm(c, p, s));
+    int flag = 0;
+    CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(c, cudaStreamSynchronize(s));
+    if (flag) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
     return BIP_OK;
 }
 
@@ -2960,8 +3012,8 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
             CUDA_TRY(c, ensure(c->g_sA2, SB * 4 * (size_t)D128 * KB * sizeof(uint16_t), true, s));
             CUDA_TRY(c, ensure(c->g_sB2, SB * 4 * (size_t)K * KB * sizeof(uint16_t), true, s));
         }
-        CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     }
+    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     CUDA_TRY(c, ensure(c->opA32, SB * perA * sizeof(float2), true, s));
     CUDA_TRY(c, ensure(c->opB32, SB * perB * sizeof(float2), true, s));
     st = operand_layout(c, K, s);
@@ -3058,47 +3110,35 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
             A.wait_ns = c->wait_ns;
             CUDA_TRY(c, bip_tc_gemm(A, s));
         } else {
-            CGemmArgs A{};
-            A.M = geo.n_det; A.N = nch * Bpad; A.K = K;
-            A.A = (const float2*)c->opA32.p; A.lda = K; A.strideA = (int64_t)perA;
-            A.Bm = (const float2*)c->opB32.p; A.ldb = K; A.strideB = (int64_t)perB;
-            A.batch = nb;
-            A.epi = 1;
-            A.C = (float2*)c->mt32.p; A.ldc = (int64_t)ldm; A.strideC = (int64_t)perMt;
-            A.ep_B = Bpad; A.ep_Dp = Dpad;
-            CUDA_TRY(c, bip_cgemm_simt(A, s));
+            CUDA_TRY(c, cgemm(c, coupling_f32(geo.n_det, nch * Bpad, K, c->opA32.p, (int64_t)perA, c->opB32.p,
+                                              (int64_t)perB, c->mt32.p, (int64_t)ldm, (int64_t)perMt, Bpad, Dpad, nb), s));
         }
         // R_tau = f o_tau sum_{rho in crop} g c c^H
         CUDA_TRY(c, bip_grad_crop_weights(gab, nb, ids, (float*)c->g_w.p, s));
-        CGemmGen r{};
-        r.M = B; r.N = B; r.K = P; r.batch = nb;
-        r.A = (const float2*)c->illum.p; r.sam = P; r.sak = 1; r.sab = 0;
+        CGemmF32 r{};
+        r.M = B; r.N = B; r.batch = nb;
+        r.A = CGemmOperand{(const float2*)c->illum.p, P, 1, 0, P, 1, 0, 0, 0};
         r.dk = (const float*)c->g_w.p; r.sdb = P;
-        r.B = (const float2*)c->illum.p; r.sbk = 1; r.sbn = P; r.sbb = 0; r.conjB = 1;
-        r.C = (float2*)c->g_R.p; r.scm = Bpad; r.scn = 1; r.scb = (int64_t)perQ;
-        CUDA_TRY(c, bip_cgemm_gen(r, s));
+        r.B = r.A;
+        r.conjB = 1;
+        r.C = (float2*)c->g_R.p; r.scm = Bpad; r.scb = (int64_t)perQ;
+        CUDA_TRY(c, cgemm(c, r, s));
         if (d_aberr) {
             // Q = sum_n M_n^H M_n, then D_b += (Q R)_bb
-            CGemmArgs Bq{};
-            Bq.M = Bpad; Bq.N = Bpad; Bq.K = (int)ldm;
-            Bq.A = (const float2*)c->mt32.p; Bq.lda = (int64_t)ldm; Bq.strideA = (int64_t)perMt;
-            Bq.Bm = Bq.A; Bq.ldb = Bq.lda; Bq.strideB = Bq.strideA;
-            Bq.conjA = 1;
-            Bq.batch = nb;
-            Bq.epi = 0;
-            Bq.C = (float2*)c->q32.p; Bq.ldc = Bpad; Bq.strideC = (int64_t)perQ;
-            CUDA_TRY(c, bip_cgemm_simt(Bq, s));
+            CUDA_TRY(c, cgemm(c, gram_f32(Bpad, (int64_t)ldm, c->mt32.p, (int64_t)perMt, c->q32.p, (int64_t)perQ, false,
+                                          nb), s));
             CUDA_TRY(c, bip_grad_aberr(B, Bpad, nb, (const float2*)c->q32.p, (int64_t)perQ, (const float2*)c->g_R.p,
                                        (int64_t)perQ, (double2*)c->g_D.p, (double2*)c->g_Dsum.p, s));
         }
         if (d_H || d_V) {
             // Mbar_n = M_n R, kept as GMt = conj(R) Mt (R Hermitian)
-            CGemmGen m{};
-            m.M = B; m.N = (int)ldm; m.K = B; m.batch = nb;
-            m.A = (const float2*)c->g_R.p; m.sam = Bpad; m.sak = 1; m.sab = (int64_t)perQ; m.conjA = 1;
-            m.B = (const float2*)c->mt32.p; m.sbk = (int64_t)ldm; m.sbn = 1; m.sbb = (int64_t)perMt;
-            m.C = (float2*)c->g_gmt.p; m.scm = (int64_t)ldm; m.scn = 1; m.scb = (int64_t)perMt;
-            CUDA_TRY(c, bip_cgemm_gen(m, s));
+            CGemmF32 m{};
+            m.M = B; m.N = (int)ldm; m.batch = nb;
+            m.A = CGemmOperand{(const float2*)c->g_R.p, Bpad, 1, (int64_t)perQ, B, 1, 0, 0, 0};
+            m.conjA = 1;
+            m.B = CGemmOperand{(const float2*)c->mt32.p, 1, (int64_t)ldm, (int64_t)perMt, B, 1, 0, 0, 0};
+            m.C = (float2*)c->g_gmt.p; m.scm = (int64_t)ldm; m.scb = (int64_t)perMt;
+            CUDA_TRY(c, cgemm(c, m, s));
             // T_n(b, r) = sum_d Mbar_n(d, b) conj S2_d(r)
             if (tcg) {
                 // B operand: conj(S2) transposed to rows r, K = d (once per batch)
@@ -3129,13 +3169,14 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
                     t.wait_ns = c->wait_ns;
                     CUDA_TRY(c, bip_tc_gemm(t, s));
                 } else {
-                    CGemmGen t{};
-                    t.M = B; t.N = K; t.K = geo.n_det; t.batch = nb;
-                    t.A = (const float2*)c->g_gmt.p + (size_t)n * Dpad; t.sam = (int64_t)ldm; t.sak = 1;
-                    t.sab = (int64_t)perMt;
-                    t.B = (const float2*)c->opA32.p; t.sbk = K; t.sbn = 1; t.sbb = (int64_t)perA; t.conjB = 1;
-                    t.C = (float2*)c->g_T.p + (size_t)n * Bpad * K; t.scm = K; t.scn = 1; t.scb = (int64_t)perT;
-                    CUDA_TRY(c, bip_cgemm_gen(t, s));
+                    CGemmF32 t{};
+                    t.M = B; t.N = K; t.batch = nb;
+                    t.A = CGemmOperand{(const float2*)c->g_gmt.p + (size_t)n * Dpad, (int64_t)ldm, 1, (int64_t)perMt,
+                                       geo.n_det, 1, 0, 0, 0};
+                    t.B = CGemmOperand{(const float2*)c->opA32.p, 1, K, (int64_t)perA, geo.n_det, 1, 0, 0, 0};
+                    t.conjB = 1;
+                    t.C = (float2*)c->g_T.p + (size_t)n * Bpad * K; t.scm = K; t.scb = (int64_t)perT;
+                    CUDA_TRY(c, cgemm(c, t, s));
                 }
             }
             if (d_H)
@@ -3176,18 +3217,14 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
                 u.wait_ns = c->wait_ns;
                 CUDA_TRY(c, bip_tc_gemm(u, s));
             } else {
-                for (int n = 0; n < nch; ++n) {
-                    CGemmGen u{};
-                    u.M = geo.n_det; u.N = K; u.K = B; u.batch = nb;
-                    u.A = (const float2*)c->g_gmt.p + (size_t)n * Dpad; u.sam = 1; u.sak = (int64_t)ldm;
-                    u.sab = (int64_t)perMt;
-                    u.B = (const float2*)c->opB32.p + (size_t)n * Bpad * K; u.sbk = K; u.sbn = 1;
-                    u.sbb = (int64_t)perB;
-                    u.conjB = 1;
-                    u.C = (float2*)c->g_s2bar.p; u.scm = K; u.scn = 1; u.scb = (int64_t)perS2bar;
-                    u.accumulate = n > 0;
-                    CUDA_TRY(c, bip_cgemm_gen(u, s));
-                }
+                // one contraction over k = (n, b), the channels as the blocks of the k axis
+                CGemmF32 u{};
+                u.M = geo.n_det; u.N = K; u.batch = nb;
+                u.A = CGemmOperand{(const float2*)c->g_gmt.p, 1, (int64_t)ldm, (int64_t)perMt, B, nch, Dpad, 0, 0};
+                u.B = CGemmOperand{(const float2*)c->opB32.p, 1, K, (int64_t)perB, B, nch, (int64_t)Bpad * K, 0, 0};
+                u.conjB = 1;
+                u.C = (float2*)c->g_s2bar.p; u.scm = K; u.scb = (int64_t)perS2bar;
+                CUDA_TRY(c, cgemm(c, u, s));
             }
             // back through the reconstructions into the window adjoints
             for (int side = 1; side <= 2; ++side) {
@@ -3220,7 +3257,7 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
             }
         }
     }
-    if (tcg) {
+    {
         int flag = 0;
         CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(c, cudaStreamSynchronize(s));
@@ -3438,7 +3475,7 @@ bip_status bip_site_coupling(bip_ctx* c, const void* H, int32_t site, void* m_ou
         g2.out_c64 = (float2*)opA.p; g2.site_stride = (int64_t)perA;
         g1.out_c64 = (float2*)opB.p; g1.site_stride = (int64_t)perB;
     }
-    if (tc) CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
+    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     if (f8) {
         bip_status st = f8_hmax(c, H, s);
         if (st != BIP_OK) return st;
@@ -3483,21 +3520,16 @@ bip_status bip_site_coupling(bip_ctx* c, const void* H, int32_t site, void* m_ou
         }
         TIMED(c, BIP_STAGE_COUPLING, s, bip_tc_gemm(A, s));
     } else {
-        CGemmArgs A{};
-        A.M = geo.n_det; A.N = (int)ldc; A.K = K;
-        A.A = (const float2*)opA.p; A.lda = K; A.strideA = (int64_t)perA;
-        A.Bm = (const float2*)opB.p; A.ldb = K; A.strideB = (int64_t)perB;
-        A.batch = 1;
-        A.epi = 0;
-        A.C = tmp; A.ldc = (int64_t)ldc; A.strideC = 0;
-        TIMED(c, BIP_STAGE_COUPLING, s, bip_cgemm_simt(A, s));
+        CGemmF32 A = coupling_f32(geo.n_det, (int)ldc, K, opA.p, (int64_t)perA, opB.p, (int64_t)perB, tmp, 0, 0, 0, 0, 1);
+        A.scm = (int64_t)ldc;
+        TIMED(c, BIP_STAGE_COUPLING, s, cgemm(c, A, s));
     }
     // [n_det][(ch, b)] -> m_out[ch][n_det][B]
     for (int ch = 0; ch < nch; ++ch)
         CUDA_TRY(c, cudaMemcpy2DAsync((float2*)m_out + (size_t)ch * geo.n_det * geo.B, geo.B * sizeof(float2),
                                       tmp + (size_t)ch * Bpad, ldc * sizeof(float2), geo.B * sizeof(float2),
                                       geo.n_det, cudaMemcpyDeviceToDevice, s));
-    if (tc) {
+    {
         int flag = 0;
         CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(c, cudaStreamSynchronize(s));

@@ -295,19 +295,34 @@ struct F8ScaleArgs {
 };
 cudaError_t bip_f8_scales(const F8ScaleArgs& a, cudaStream_t s);
 
-// gemm_simt.cu : FP32 complex GEMMs, C[m][n] = sum_k op(A[m][k]) B[n][k]
-struct CGemmArgs {
-    int M, N, K;                    // complex sizes (K multiple of 16)
-    const float2* A; int64_t lda, strideA;   // row-major [M][lda], batch stride
-    const float2* Bm; int64_t ldb, strideB;
-    int conjA;
-    int batch;
-    // epilogue
-    int epi;                        // 0: C row-major; 1: transposed to Mt[n%Bp][(n/Bp)*Dp + m]
-    float2* C; int64_t ldc, strideC;
-    int ep_B, ep_Dp;                // epilogue 1 geometry
+// cgemm_f32.cu : FP32 complex contractions on tcgen05 (three BF16 terms per
+// element), C(m, n) = sum_k opA(A(m, k) dk[k]) opB(B(k, n)) per batch
+struct CGemmOperand {
+    const float2* p;
+    int64_t sr, sk, sb;             // strides of a row (m or n), of k, of the batch; sr or sk is 1
+    int kvalid;                     // k's of one block of the k axis
+    int nper; int64_t sk2;          // blocks of the k axis and their stride (1, 0: one block)
+    int kper, vec;                  // (plan) kvalid rounded up to whole chunks; 16-byte loads
 };
-cudaError_t bip_cgemm_simt(const CGemmArgs& a, cudaStream_t s);
+struct CGemmF32 {
+    int M, N, batch;
+    CGemmOperand A, B;
+    int conjA, conjB;
+    const float* dk; int64_t sdb;   // optional real scale of each k (null: 1), with one k block only
+    // C(m, n) at C[z scb + m scm + n], or with ep_B > 0 (n = (ch, b)) at
+    // C[z scb + b scn + ch ep_Dp + m]
+    float2* C; int64_t scm, scn, scb;
+    int ep_B, ep_Dp;
+    int tri;                        // only the column tiles that reach the diagonal or lie right of it
+    float2* part;                   // workspace of a split k range
+    int* err;
+    uint64_t wait_ns;
+    // (plan)
+    int nt, n_tiles, tiles, steps, ksplit, units, vecC;
+};
+// fills the plan; *part_elems: float2 elements `part` must hold (0: none)
+cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems);
+cudaError_t bip_cgemm_f32(const CGemmF32& p, cudaStream_t s);
 
 // difftrans.cu : the per-site quadratic form c^H Q c as a trigonometric
 // polynomial over beam-lattice differences (see the file's header)
@@ -562,17 +577,6 @@ cudaError_t bip_s1bar(int nb, const int32_t* ids, const SiteDev* sites, int B, i
                       const float2* T, int64_t t_site, int64_t t_ch, float2* S1bar, int64_t s1_site, cudaStream_t s);
 
 // grad.cu : reverse pass of a map loss through the contraction
-// generic complex GEMM: C(m, n) (+)= sum_k opA(A(m, k) dk[k]) opB(B(k, n)),
-// X(i, j) = X[z sXb + i sXi + j sXj] for batch z
-struct CGemmGen {
-    int M, N, K, batch;
-    const float2* A; int64_t sam, sak, sab;
-    const float2* B; int64_t sbk, sbn, sbb;
-    float2* C; int64_t scm, scn, scb;
-    const float* dk; int64_t sdb;   // optional real scale of each k (null: 1)
-    int conjA, conjB, accumulate;
-};
-cudaError_t bip_cgemm_gen(const CGemmGen& a, cudaStream_t s);
 struct GradArgs {
     int P, K, B;
     const double* scans;            // [P][2] pixels (device)

@@ -1,7 +1,7 @@
 // Reverse pass of a map loss through the contraction (the matrices as a
 // forward model, Sec. 5): given g(rho) = dL/dI(rho), the derivatives with
 // respect to the site occupancies, the transition potentials H and the
-// probe aberrations.  FP32 SIMT kernels; per site tau, f = f_y f_x:
+// probe aberrations.  Per site tau, f = f_y f_x:
 //   R_tau     = f o_tau sum_{rho in crop} g(rho) c(rho) c(rho)^H     [B x B]
 //   Mbar_n    = M_n R_tau            (stored as GMt = conj(R) Mt, Mt[b][(n, d)])
 //   T_n(b, r) = sum_d Mbar_n(d, b) conj S2_d(r)
@@ -9,8 +9,7 @@
 //   D_b      += (Q_tau R_tau)_bb,  dL/dtheta = -2 sum_b chi'_b Im D_b
 //   dL/do_tau = sum_rho g(rho) I_tau(rho)
 //
-//   cgemm_gen_kernel : C(m, n) (+)= sum_k opA(A(m, k) s_k) opB(B(k, n)),
-//                      arbitrary strides, batched, 64 x 64 tiles
+// The contractions run in cgemm_f32.cu (or gemm_tc.cu in split BF16); here:
 //   crop_weight_kernel, hgrad_kernel, aberr_kernel, aberr_sum_kernel,
 //   occ_grad_kernel
 #include "bip_device.cuh"
@@ -19,87 +18,9 @@
 
 namespace {
 
-constexpr int kTile = 64, kKt = 16, kThreads = 256;
+constexpr int kThreads = 256;
 
 __device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
-
-__global__ void __launch_bounds__(kThreads) cgemm_gen_kernel(CGemmGen a) {
-    __shared__ float2 As[kKt][kTile + 1];
-    __shared__ float2 Bs[kKt][kTile + 1];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile, z = blockIdx.z;
-    const float2* A = a.A + (int64_t)z * a.sab;
-    const float2* B = a.B + (int64_t)z * a.sbb;
-    const float* dk = a.dk ? a.dk + (int64_t)z * a.sdb : nullptr;
-    float2 acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
-    for (int k0 = 0; k0 < a.K; k0 += kKt) {
-#pragma unroll
-        for (int l = 0; l < 4; ++l) {
-            const int idx = threadIdx.x + l * kThreads;
-            // the unit-stride axis runs fastest across the threads
-            int m, k;
-            if (a.sam == 1) { m = idx % kTile; k = idx / kTile; } else { k = idx % kKt; m = idx / kKt; }
-            float2 v = make_float2(0.f, 0.f);
-            if (m0 + m < a.M && k0 + k < a.K) {
-                v = A[(int64_t)(m0 + m) * a.sam + (int64_t)(k0 + k) * a.sak];
-                if (a.conjA) v.y = -v.y;
-                if (dk) {
-                    const float s = dk[k0 + k];
-                    v.x *= s;
-                    v.y *= s;
-                }
-            }
-            As[k][m] = v;
-            int n;
-            if (a.sbn == 1) { n = idx % kTile; k = idx / kTile; } else { k = idx % kKt; n = idx / kKt; }
-            float2 w = make_float2(0.f, 0.f);
-            if (n0 + n < a.N && k0 + k < a.K) {
-                w = B[(int64_t)(k0 + k) * a.sbk + (int64_t)(n0 + n) * a.sbn];
-                if (a.conjB) w.y = -w.y;
-            }
-            Bs[k][n] = w;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < kKt; ++k) {
-            float2 av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = As[k][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    acc[i][j].x = fmaf(av[i].x, bv[j].x, fmaf(-av[i].y, bv[j].y, acc[i][j].x));
-                    acc[i][j].y = fmaf(av[i].x, bv[j].y, fmaf(av[i].y, bv[j].x, acc[i][j].y));
-                }
-        }
-        __syncthreads();
-    }
-    float2* C = a.C + (int64_t)z * a.scb;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty + 16 * i;
-        if (m >= a.M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tx + 16 * j;
-            if (n >= a.N) continue;
-            float2* o = C + (int64_t)m * a.scm + (int64_t)n * a.scn;
-            if (a.accumulate) {
-                const float2 p = *o;
-                *o = make_float2(p.x + acc[i][j].x, p.y + acc[i][j].y);
-            } else {
-                *o = acc[i][j];
-            }
-        }
-    }
-}
 
 // w[bs][rho] = f o_tau g(rho) inside the site's crop window, else 0
 __global__ void crop_weight_kernel(GradArgs a, int nb, const int32_t* ids, float* w) {
@@ -229,14 +150,6 @@ cudaError_t bip_split_planes(const SplitArgs& a, cudaStream_t s) {
     const dim3 grid((a.cols + 31) / 32, (a.rows + 31) / 32, a.batch);
     if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
     split_planes_kernel<<<grid, dim3(32, 8), 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t bip_cgemm_gen(const CGemmGen& a, cudaStream_t s) {
-    if (a.M < 1 || a.N < 1 || a.K < 1 || a.batch < 1) return cudaErrorInvalidValue;
-    const dim3 grid((a.N + kTile - 1) / kTile, (a.M + kTile - 1) / kTile, a.batch);
-    if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
-    cgemm_gen_kernel<<<grid, kThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
