@@ -960,6 +960,7 @@ void release_map_workspaces(bip_ctx* c, cudaStream_t s) {
 // range, the launch.
 cudaError_t cgemm(bip_ctx* c, CGemmF32 p, cudaStream_t s) {
     size_t part = 0;
+    if (c->n_sites > 0) p.plan_batch = std::min(c->n_sites, 8);
     cudaError_t e = bip_cgemm_plan(p, &part);
     if (e != cudaSuccess) return e;
     if (part > 0) {

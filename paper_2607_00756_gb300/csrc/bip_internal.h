@@ -314,6 +314,7 @@ struct CGemmF32 {
     float2* C; int64_t scm, scn, scb;
     int ep_B, ep_Dp;
     int tri;                        // only the column tiles that reach the diagonal or lie right of it
+    int plan_batch;                 // batch size the k split is chosen for (0: batch)
     float2* part;                   // workspace of a split k range
     int* err;
     uint64_t wait_ns;

@@ -565,7 +565,9 @@ bool aligned2(const void* q, int64_t a, int64_t b, int64_t c) {
 // The column tile is the narrowest multiple of 8 that keeps the tile count of
 // 128-wide ones (no work for padding columns beyond 7).  The split: the parts
 // that minimise rounds x (chunks per part + the pipeline's fill, about three
-// chunks), plus the parts' way through memory at about 2.5 KB per clock.
+// chunks), plus the parts' way through memory at about 2.5 KB per clock.  It
+// is chosen for plan_batch entries, so that a site's sums do not depend on
+// how full its batch is.
 cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
     if (p.M < 1 || p.N < 1 || p.batch < 1) return cudaErrorInvalidValue;
     for (CGemmOperand* o : {&p.A, &p.B}) {
@@ -587,11 +589,12 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
     p.tiles = 0;
     for (int mt = 0; mt < m_tiles; ++mt) p.tiles += p.n_tiles - (p.tri ? mt * 128 / p.nt : 0);
     p.steps = p.A.nper * (p.A.kper / kStep);
-    const int64_t units = (int64_t)p.tiles * p.batch;
-    if (units > (1 << 26)) return cudaErrorInvalidValue;
+    const int pb = p.plan_batch > 0 ? p.plan_batch : p.batch;
+    const int64_t units = (int64_t)p.tiles * pb;
+    if (units * 16 > (1 << 26) || (int64_t)p.tiles * p.batch * 16 > (1 << 26)) return cudaErrorInvalidValue;
     const int sms = num_sms();
     const double chunk = 12.0 * p.nt;                          // clocks of a chunk's MMAs
-    const double bytes = 8.0 * p.batch * (double)p.M * p.N;
+    const double bytes = 8.0 * pb * (double)p.M * p.N;
     double best = 0.0;
     p.ksplit = 1;
     for (int S = 1; S <= 16 && S * 4 <= p.steps; ++S) {
@@ -603,7 +606,7 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
             p.ksplit = S;
         }
     }
-    p.units = (int)(units * p.ksplit);
+    p.units = p.tiles * p.batch * p.ksplit;
     *part_elems = p.ksplit > 1 ? (size_t)p.ksplit * p.batch * p.M * p.N : 0;
     return cudaSuccess;
 }
