@@ -1099,9 +1099,14 @@ bip_status recon_tc_batch(bip_ctx* c, const int32_t* ids, int nb, const void* H,
     r.stash_win = g.win;
     r.wo = (g.win - w) / 2;
     // work units of the largest multiple of 64 pixels up to 1024 that divides K
+    // and gives every SM a unit (4 sites: 48 units of 1024 pixels, 192 of 256);
+    // units of 64 pixels pay their table loads for one tile, so 128 at least
+    // -- for the call's sites, not the batch's, so that a site's re-tilt steps
+    // do not depend on how the sites are batched
+    const int64_t per_px = (int64_t)c->n_sites * (Dw / 128 + Bpad / 128) * K;
     r.chunk_px = 64;
     for (int cp = std::min(K, 1024) / 64 * 64; cp >= 64; cp -= 64)
-        if (K % cp == 0) {
+        if (K % cp == 0 && (per_px / cp >= 152 || cp <= 128)) {
             r.chunk_px = cp;
             break;
         }
@@ -1456,6 +1461,7 @@ bip_status check_map_args(bip_ctx* c, const void* H, const double* scans, int32_
 // equal y, the x of every row the same sequence (equal within 1e-9 px).
 struct Raster {
     bool ok = false;
+    bool exact = true;              // equal to the bit
     int My = 0, Mx = 0;
 };
 Raster detect_raster(const double* sc, int P) {
@@ -1469,6 +1475,7 @@ Raster detect_raster(const double* sc, int P) {
         const int i = p / Mx, j = p % Mx;
         if (std::fabs(sc[2 * p] - sc[2 * (size_t)i * Mx]) > 1e-9 || std::fabs(sc[2 * p + 1] - sc[2 * j + 1]) > 1e-9)
             return r;
+        r.exact = r.exact && sc[2 * p] == sc[2 * (size_t)i * Mx] && sc[2 * p + 1] == sc[2 * j + 1];
     }
     r.ok = true;
     r.My = My;
@@ -1523,14 +1530,31 @@ CubeArgs cube_args(const bip_ctx* c, const int32_t* ids, int nb, int P, float* c
 // Dpad / Bpad) must read as zero: the Gram contraction runs over every
 // detector row (and the probe order's operands are cleared with them).  The buffers are zeroed when allocated and every writer
 // packs target rows only, at pitch K = w^2; after a batch packed at another
-// pitch, rows that are padding at pitch K may hold values, so the buffers
-// are cleared before the pitch changes (never while every site has the
-// context's window).
+// pitch, rows that are padding at pitch K may hold values, so the padding
+// rows are cleared before the pitch changes (never while every site has the
+// context's window); clearing the whole operands took 0.92 of a 6.5 ms map
+// of 48 sites with two window sizes.
 bip_status operand_layout(bip_ctx* c, int K, cudaStream_t s) {
     if (c->op_k == K) return BIP_OK;
-    if (c->op_k != 0)
-        for (DevBuf* b : {&c->opA16, &c->opB16, &c->op8A, &c->op8B, &c->opA32, &c->opB32, &c->s1t, &c->psi, &c->ybuf})
+    if (c->op_k != 0) {
+        // the coupling's operands: planes of Dpad (detector) or Bpad (aperture)
+        // rows, their last Dpad - n_det or Bpad - B rows padding
+        struct Op {
+            DevBuf* b;
+            int rows, used;
+            size_t elem;
+        };
+        const int nd = c->geo.n_det, nb = c->geo.B;
+        for (const Op& o : {Op{&c->opA16, c->Dpad, nd, 2}, Op{&c->opB16, c->Bpad, nb, 2}, Op{&c->op8A, c->Dpad, nd, 1},
+                            Op{&c->op8B, c->Bpad, nb, 1}, Op{&c->opA32, c->Dpad, nd, 8}, Op{&c->opB32, c->Bpad, nb, 8}}) {
+            const size_t row = (size_t)K * o.elem, plane = o.rows * row;
+            if (!o.b->p || o.used == o.rows || o.b->cap < plane) continue;
+            CUDA_TRY(c, cudaMemset2DAsync((char*)o.b->p + o.used * row, plane, 0, (o.rows - o.used) * row,
+                                          o.b->cap / plane, s));
+        }
+        for (DevBuf* b : {&c->s1t, &c->psi, &c->ybuf})
             if (b->p) CUDA_TRY(c, cudaMemsetAsync(b->p, 0, b->cap, s));
+    }
     c->op_k = K;
     return BIP_OK;
 }
@@ -1637,7 +1661,7 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
             CUDA_TRY(c, upload(c->ray, ay, s));
             CUDA_TRY(c, upload(c->rax, ax, s));
         }
-        rargs = RasterArgs{raster.My, raster.Mx, (const float2*)c->ray.p, (const float2*)c->rax.p};
+        rargs = RasterArgs{raster.My, raster.Mx, (const float2*)c->ray.p, (const float2*)c->rax.p, raster.exact ? 1 : 0};
     }
 
     // scan-tile bounding boxes (host)

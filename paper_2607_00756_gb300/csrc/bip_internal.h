@@ -360,6 +360,7 @@ struct RasterArgs {
     int My, Mx;
     const float2* Ay;
     const float2* Ax;
+    int exact;                      // every row's y and every column's x bit for bit the same
 };
 cudaError_t bip_raster_eval(const DiffArgs& a, const RasterArgs& r, cudaStream_t s);
 

@@ -58,19 +58,33 @@ __global__ void __launch_bounds__(kBinWarps * 32) diff_bin_kernel(DiffArgs a) {
     const float2* Q = a.Q + (size_t)bs * a.q_site;
     float gr = 0.f, gi = 0.f;
     if (dy < 0 || dx <= 0) {
-        for (int b = lane; b < a.B; b += 32) {
-            const int2 k = kb[b];
-            const int ky = k.x - dy, kx = k.y - dx;          // partner k_b' = k_b - Delta
-            if (ky < -a.Ky || ky > a.Ky || kx < -a.Kx || kx > a.Kx) continue;
-            const int bp = lat[(ky + a.Ky) * lw + kx + a.Kx];
-            if (bp < 0) continue;
-            const float2 q = __ldg(&Q[(size_t)b * a.ldq + bp]);
-            const float2 cb = cf[b], cp = cf[bp];
-            // w conj(c_b) q c_b', w = 1 on the diagonal, 2 above it
-            const float w = (bp == b) ? 1.f : 2.f;
-            const float2 t = c_mul(make_float2(cb.x, -cb.y), c_mul(q, cp));
-            gr = fmaf(w, t.x, gr);
-            gi = fmaf(w, t.y, gi);
+        // four beams of the lane at a time, their Q in flight together (the
+        // scattered loads' latency is what the pass waits for)
+        for (int b0 = lane; b0 < a.B; b0 += 128) {
+            float2 q[4];
+            int bp[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int b = b0 + 32 * i;
+                bp[i] = -1;
+                if (b >= a.B) continue;
+                const int2 k = kb[b];
+                const int ky = k.x - dy, kx = k.y - dx;      // partner k_b' = k_b - Delta
+                if (ky < -a.Ky || ky > a.Ky || kx < -a.Kx || kx > a.Kx) continue;
+                bp[i] = lat[(ky + a.Ky) * lw + kx + a.Kx];
+                if (bp[i] >= 0) q[i] = __ldg(&Q[(size_t)b * a.ldq + bp[i]]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (bp[i] < 0) continue;
+                const int b = b0 + 32 * i;
+                const float2 cb = cf[b], cp = cf[bp[i]];
+                // w conj(c_b) q c_b', w = 1 on the diagonal, 2 above it
+                const float w = (bp[i] == b) ? 1.f : 2.f;
+                const float2 t = c_mul(make_float2(cb.x, -cb.y), c_mul(q[i], cp));
+                gr = fmaf(w, t.x, gr);
+                gi = fmaf(w, t.y, gi);
+            }
         }
     }
 #pragma unroll
@@ -140,21 +154,35 @@ __global__ void __launch_bounds__(256) diff_eval_kernel(DiffArgs a) {
     }
 }
 
-// Raster scans: block = (64 scan rows, site), four warps of 16 rows each;
+// Raster scans: block = (4 WR scan rows, site), four warps of WR rows each;
 // stage 1 Y[r][j] = sum_iy Ay[my][iy] G[iy][j] for the block's rows into
-// shared memory, stage 2 lane = four adjacent scan columns, 16 rows x 4
+// shared memory, stage 2 lane = CX adjacent scan columns, WR rows x CX
 // columns of Re(Y Ax) per thread (Ax[j][.] loaded once per j and lane).
-constexpr int kRasterWarpRows = 16;
-constexpr int kRasterRows = 4 * kRasterWarpRows;
+// The crop mask is a product over the axes, so the block tests its rows and
+// the columns once (FP64) instead of every scan: those tests, at GB300's low
+// FP64 rate, took most of the kernel.
+constexpr int kRasterFlags = 16384;        // columns the block keeps a crop flag for, at most
+template <int WR, int CX>
 __global__ void __launch_bounds__(128) raster_eval_kernel(DiffArgs a, RasterArgs r) {
+    constexpr int BR = 4 * WR;
     extern __shared__ float2 rs[];
     const int rows = 2 * a.Ky + 1, cols = 4 * a.Kx + 1;
     const int nd = rows * cols;
     float2* gs = rs;                       // [rows][cols]
-    float2* ys = rs + nd;                  // [kRasterRows][cols]
+    float2* ys = rs + nd;                  // [BR][cols]
+    uint8_t* cy = reinterpret_cast<uint8_t*>(ys + BR * cols);   // [BR] rows inside the crop
+    uint8_t* cx = cy + BR;                                      // [Mx] columns inside it
     const int bs = blockIdx.y;
-    const int my0 = blockIdx.x * kRasterRows;
-    const int nr = min(kRasterRows, r.My - my0);
+    const int my0 = blockIdx.x * BR;
+    const int nr = min(BR, r.My - my0);
+    const int site = a.site_ids[bs];
+    const SiteDev st = a.sites[site];
+    if (r.exact) {
+        for (int i = threadIdx.x; i < nr; i += blockDim.x)
+            cy[i] = in_crop_axis(a.scans[2 * (size_t)(my0 + i) * r.Mx], st.ty, a.ny, a.fy);
+        for (int i = threadIdx.x; i < r.Mx; i += blockDim.x)
+            cx[i] = in_crop_axis(a.scans[2 * i + 1], st.tx, a.nx, a.fx);
+    }
     for (int i = threadIdx.x; i < nd; i += blockDim.x) gs[i] = a.G[(size_t)bs * nd + i];
     __syncthreads();
     for (int i = threadIdx.x; i < nr * cols; i += blockDim.x) {
@@ -170,57 +198,74 @@ __global__ void __launch_bounds__(128) raster_eval_kernel(DiffArgs a, RasterArgs
     }
     __syncthreads();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int q0 = warp * kRasterWarpRows;                 // this warp's first row in the block
-    const int wr = min(kRasterWarpRows, nr - q0);          // its rows (may be <= 0)
+    const int q0 = warp * WR;                              // this warp's first row in the block
+    const int wr = min(WR, nr - q0);                       // its rows (may be <= 0)
     if (wr <= 0) return;
-    const int site = a.site_ids[bs];
-    const SiteDev st = a.sites[site];
-    for (int mx0 = 4 * lane; mx0 < r.Mx; mx0 += 128) {
-        float acc[kRasterWarpRows][4];
+    for (int mx0 = CX * lane; mx0 < r.Mx; mx0 += 32 * CX) {
+        float acc[WR][CX];
 #pragma unroll
-        for (int q = 0; q < kRasterWarpRows; ++q)
+        for (int q = 0; q < WR; ++q)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc[q][k] = 0.f;
+            for (int k = 0; k < CX; ++k) acc[q][k] = 0.f;
         for (int j = 0; j < cols; ++j) {
-            float2 x[4];
+            float2 x[CX];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) x[k] = mx0 + k < r.Mx ? __ldg(&r.Ax[(size_t)j * r.Mx + mx0 + k]) : make_float2(0.f, 0.f);
+            for (int k = 0; k < CX; ++k) x[k] = mx0 + k < r.Mx ? __ldg(&r.Ax[(size_t)j * r.Mx + mx0 + k]) : make_float2(0.f, 0.f);
 #pragma unroll
-            for (int q = 0; q < kRasterWarpRows; ++q) {
+            for (int q = 0; q < WR; ++q) {
                 const float2 y = ys[(q0 + (q < wr ? q : 0)) * cols + j];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[q][k] = fmaf(y.x, x[k].x, fmaf(-y.y, x[k].y, acc[q][k]));   // Re(y x)
+                for (int k = 0; k < CX; ++k) acc[q][k] = fmaf(y.x, x[k].x, fmaf(-y.y, x[k].y, acc[q][k]));   // Re(y x)
             }
         }
-        for (int q = 0; q < wr; ++q) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+        for (int q = 0; q < WR; ++q) {
+            if (q >= wr) continue;
+#pragma unroll
+            for (int k = 0; k < CX; ++k) {
                 const int mx = mx0 + k;
                 if (mx >= r.Mx) continue;
                 const int n = (my0 + q0 + q) * r.Mx + mx;
-                if (in_crop(a.scans[2 * n], a.scans[2 * n + 1], st.ty, st.tx, a.ny, a.nx, a.fy, a.fx))
-                    a.partial[(size_t)site * a.P + n] = a.scale * acc[q][k];
+                const bool in = r.exact ? cy[q0 + q] && cx[mx]
+                                        : in_crop(a.scans[2 * n], a.scans[2 * n + 1], st.ty, st.tx, a.ny, a.nx, a.fy, a.fx);
+                if (in) a.partial[(size_t)site * a.P + n] = a.scale * acc[q][k];
             }
         }
     }
 }
 
-}  // namespace
-
-cudaError_t bip_raster_eval(const DiffArgs& a, const RasterArgs& r, cudaStream_t s) {
-    if (a.n_sites < 1 || r.My < 1 || r.Mx < 1 || (int64_t)r.My * r.Mx != a.P) return cudaErrorInvalidValue;
+template <int WR, int CX>
+cudaError_t launch_raster(const DiffArgs& a, const RasterArgs& r, cudaStream_t s) {
+    constexpr int BR = 4 * WR;
     const size_t nd = (size_t)(2 * a.Ky + 1) * (4 * a.Kx + 1);
-    const size_t sm = (nd + (size_t)kRasterRows * (4 * a.Kx + 1)) * sizeof(float2);
-    if (sm > 200 * 1024) return cudaErrorInvalidValue;
+    const size_t sm = (nd + (size_t)BR * (4 * a.Kx + 1)) * sizeof(float2) + (r.exact ? BR + r.Mx : 0);
     static std::atomic<size_t> attr{0};
     if (sm > 48 * 1024) {
         const cudaError_t e = bip_raise_once(attr, sm, [&] {
-            return cudaFuncSetAttribute(raster_eval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            return cudaFuncSetAttribute(raster_eval_kernel<WR, CX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         });
         if (e != cudaSuccess) return e;
     }
-    raster_eval_kernel<<<dim3((r.My + kRasterRows - 1) / kRasterRows, a.n_sites), 128, sm, s>>>(a, r);
+    raster_eval_kernel<WR, CX><<<dim3((r.My + BR - 1) / BR, a.n_sites), 128, sm, s>>>(a, r);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+// Blocks of 64 rows where they fill the chip twice over (1600 sites x 128 x
+// 128: two per site); fewer rows per block below that (4 sites x 16 x 16
+// scans ran as four blocks of one busy warp), and one column per lane on
+// narrow rasters, whose rows would leave most lanes idle at four.
+// Rasters that are not exact to the bit, or too wide for the column flags,
+// keep the per-scan test.
+cudaError_t bip_raster_eval(const DiffArgs& a, const RasterArgs& raster, cudaStream_t s) {
+    RasterArgs r = raster;
+    if (a.n_sites < 1 || r.My < 1 || r.Mx < 1 || (int64_t)r.My * r.Mx != a.P) return cudaErrorInvalidValue;
+    const size_t cols = 4 * a.Kx + 1;
+    if (((size_t)(2 * a.Ky + 1) + 64) * cols * sizeof(float2) > 200 * 1024) return cudaErrorInvalidValue;
+    if (r.Mx > kRasterFlags) r.exact = 0;
+    if ((int64_t)((r.My + 63) / 64) * a.n_sites >= 2 * 152) return launch_raster<16, 4>(a, r, s);
+    return r.Mx > 64 ? launch_raster<4, 4>(a, r, s) : launch_raster<4, 1>(a, r, s);
 }
 
 cudaError_t bip_diff_bin(const DiffArgs& a, cudaStream_t s) {
