@@ -367,6 +367,26 @@ std::vector<double2> coef_host(const bip_ctx* c) {
     return coef;
 }
 
+// Separable propagator exp(-i pi lambda dz q^2) per axis, with the 1/(ny nx)
+// of the unnormalised inverse FFTs folded in: 1/n in each axis' table, or, in
+// contexts made for FP32, both in the first.  On 3 x 2^k grids that rounds 1/9
+// once (+7e-9 at the zero beam, every slice) instead of 1/3 twice (+6e-8: 1.5e-6
+// of an FP32 map after 25 slices of 384^2); power-of-two grids have the same
+// bits either way, and the narrower precisions, whose roundings a last bit can
+// move (E4M3: 4e-5 of a map), keep theirs.
+void propagator_tables(const bip_config& g, double lambda, std::vector<float2>& py, std::vector<float2>& px) {
+    const bool first = g.prec == BIP_PREC_FP32;
+    auto axis = [&](std::vector<float2>& p, int n, double l, double norm) {
+        for (int k = 0; k < n; ++k) {
+            const double q = signed_bin(k, n) / l;
+            const double a = -kPi * lambda * g.dz * q * q;
+            p[k] = float2{(float)(std::cos(a) / norm), (float)(std::sin(a) / norm)};
+        }
+    };
+    axis(py, g.ny, g.ly, first ? (double)g.ny * g.nx : g.ny);
+    axis(px, g.nx, g.lx, first ? 1.0 : g.nx);
+}
+
 bip_status make_tables(bip_ctx* c, cudaStream_t s) {
     if (c->tables) return BIP_OK;
     const bip_config& g = c->cfg;
@@ -379,22 +399,7 @@ bip_status make_tables(bip_ctx* c, cudaStream_t s) {
     std::vector<float2> ey(g.ny), ex(g.nx), py(g.ny), px(g.nx);
     for (int m = 0; m < g.ny; ++m) ey[m] = turn(m, g.ny, +1.0);
     for (int m = 0; m < g.nx; ++m) ex[m] = turn(m, g.nx, +1.0);
-    // separable propagator exp(-i pi lambda dz q^2) per axis, with the 1/(ny nx)
-    // of the unnormalised inverse FFTs folded into the first.  One rounding of
-    // 1/9 on 3 x 2^k grids (+7e-9 at the zero beam, every slice) instead of two
-    // of 1/3 (+6e-8: 1.5e-6 of a map after 25 slices of 384^2); the same bits on
-    // power-of-two grids.
-    const double norm = (double)g.ny * g.nx;
-    for (int k = 0; k < g.ny; ++k) {
-        const double q = signed_bin(k, g.ny) / g.ly;
-        const double a = -kPi * geo.lambda * g.dz * q * q;
-        py[k] = float2{(float)(std::cos(a) / norm), (float)(std::sin(a) / norm)};
-    }
-    for (int k = 0; k < g.nx; ++k) {
-        const double q = signed_bin(k, g.nx) / g.lx;
-        const double a = -kPi * geo.lambda * g.dz * q * q;
-        px[k] = float2{(float)std::cos(a), (float)std::sin(a)};
-    }
+    propagator_tables(g, geo.lambda, py, px);
     std::vector<int2> sh1(geo.Bp1), sh2(geo.Bp2), hb(geo.B), hd(geo.n_det);
     for (int i = 0; i < geo.Bp1; ++i) sh1[i] = int2{geo.h_beam[2 * geo.p1[i]], geo.h_beam[2 * geo.p1[i] + 1]};
     for (int i = 0; i < geo.Bp2; ++i) sh2[i] = int2{-geo.h_det[2 * geo.p2[i]], -geo.h_det[2 * geo.p2[i] + 1]};
@@ -1102,11 +1107,12 @@ bip_status recon_tc_batch(bip_ctx* c, const int32_t* ids, int nb, const void* H,
     // and gives every SM a unit (4 sites: 48 units of 1024 pixels, 192 of 256);
     // units of 64 pixels pay their table loads for one tile, so 128 at least
     // -- for the call's sites, not the batch's, so that a site's re-tilt steps
-    // do not depend on how the sites are batched
+    // do not depend on how the sites are batched; E4M3 rows, which a last bit of
+    // the re-tilt can move by a step, keep the longest
     const int64_t per_px = (int64_t)c->n_sites * (Dw / 128 + Bpad / 128) * K;
     r.chunk_px = 64;
     for (int cp = std::min(K, 1024) / 64 * 64; cp >= 64; cp -= 64)
-        if (K % cp == 0 && (per_px / cp >= 152 || cp <= 128)) {
+        if (K % cp == 0 && (per_px / cp >= 152 || cp <= 128 || f8)) {
             r.chunk_px = cp;
             break;
         }
@@ -3619,17 +3625,7 @@ extern "C" bip_status bip_build_s1_noalloc(bip_ctx* c, const float* V, const bip
     // host tables (same definitions as the context's: FP64 then rounded)
     const std::vector<float2> twy = fft_twiddles(g.ny), twx = fft_twiddles(g.nx);
     std::vector<float2> py(g.ny), px(g.nx);
-    const double norm = (double)g.ny * g.nx;
-    for (int k = 0; k < g.ny; ++k) {
-        const double q = signed_bin(k, g.ny) / g.ly;
-        const double a = -kPi * geo.lambda * g.dz * q * q;
-        py[k] = float2{(float)(std::cos(a) / norm), (float)(std::sin(a) / norm)};
-    }
-    for (int k = 0; k < g.nx; ++k) {
-        const double q = signed_bin(k, g.nx) / g.lx;
-        const double a = -kPi * geo.lambda * g.dz * q * q;
-        px[k] = float2{(float)std::cos(a), (float)std::sin(a)};
-    }
+    propagator_tables(g, geo.lambda, py, px);
     std::vector<int2> sh(ncol);
     for (int i = 0; i < ncol; ++i) sh[i] = int2{geo.h_beam[2 * geo.p1[i]], geo.h_beam[2 * geo.p1[i] + 1]};
     // planes that hold sites
