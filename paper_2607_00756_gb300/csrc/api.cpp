@@ -3186,20 +3186,23 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
                     SplitArgs sg{(const float2*)c->g_gmt.p + (size_t)n * Dpad, (int64_t)ldm, 1, (int64_t)perMt, Bpad,
                                  Dpad, nb, (uint16_t*)c->g_tA.p, (int64_t)4 * Bpad * Dpad, Bpad, Dpad, 0, 0};
                     CUDA_TRY(c, bip_split_planes(sg, s));
+                    // the pixels as the tiles' rows, the beams (16-padded, where rows
+                    // would be padded to 128) as their columns
                     TcArgs t{};
                     t.epi = TC_EPI_C32;
-                    t.N = 256;
+                    t.n_cols = round_up(B, 16);
+                    t.N = tile_width(t.n_cols);
                     t.npl = 4;
-                    t.A = TcOperand{c->g_tA.p, (int64_t)nb * 4 * Bpad, Dpad, 4 * (int64_t)Bpad, Bpad};
-                    t.B = TcOperand{c->g_tB.p, (int64_t)nb * 4 * K, Dpad, 4 * (int64_t)K, K};
+                    t.A = TcOperand{c->g_tB.p, (int64_t)nb * 4 * K, Dpad, 4 * (int64_t)K, K};
+                    t.B = TcOperand{c->g_tA.p, (int64_t)nb * 4 * Bpad, Dpad, 4 * (int64_t)Bpad, Bpad};
                     t.kb = Dpad / 32;
                     t.n_sites = nb;
-                    t.mt_per = Bpad / 128;
-                    t.nt_per = (K + 255) / 256;
-                    t.n_cols = K;
+                    t.mt_per = K / 128;
+                    t.nt_per = (t.n_cols + t.N - 1) / t.N;
                     t.out32 = (float2*)c->g_T.p + (size_t)n * Bpad * K;
                     t.out32_site = (int64_t)perT;
                     t.out32_ld = K;
+                    t.out32_trans = 1;
                     t.err = (int*)c->errflag.p;
                     t.wait_ns = c->wait_ns;
                     CUDA_TRY(c, bip_tc_gemm(t, s));
@@ -3286,6 +3289,10 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
                     ra.Sbar = (const float2*)c->g_s2bar.p; ra.sbar_rows = (int)(perS2bar / K);
                     ra.dtbar = (float2*)c->g_dt2.p;
                 }
+                ra.ey = (const float2*)c->ey.p;
+                ra.ex = (const float2*)c->ex.p;
+                ra.ytab = (const float2*)c->ytab.p;
+                ra.xtab = (const float2*)c->xtab.p;
                 ra.Ubar = (float2*)c->g_ubar.p;
                 ra.dA = (float*)c->g_dA.p;
                 CUDA_TRY(c, bip_recon_adjoint(ra, s));

@@ -569,6 +569,10 @@ struct ReconAdjArgs {
     AdjWeights w;
     const float2* Sbar;             // [bs][rows][K] dL/dS*, row stride sbar_rows
     int sbar_rows;
+    const float2* ey;               // re-tilt tables, as GatherArgs'
+    const float2* ex;
+    const float2* ytab;
+    const float2* xtab;
     float2* Ubar;                   // scratch [bs][n_targets][K]
     float* dA;                      // scratch [bs][n_targets][K]
     float2* dtbar;                  // out [n_sites_total][Bp][stash_win^2]: the batch's sites' blocks

@@ -48,6 +48,7 @@ __global__ void hgrad_kernel(GradArgs a, const int32_t* ids, const float2* S1, i
     const float2* s1 = S1 + (int64_t)bs * s1_site + r;
     const float2* t = T + (int64_t)bs * t_site + (int64_t)n * t_ch + r;
     float2 acc = make_float2(0.f, 0.f);
+#pragma unroll 8                     // eight beams' loads in flight: few blocks, a long sum each
     for (int b = 0; b < a.B; ++b) {
         const float2 x = conjf2(__ldg(&s1[(int64_t)b * a.K]));
         const float2 y = __ldg(&t[(int64_t)b * a.K]);
