@@ -104,10 +104,12 @@ struct bip_ctx {
     bool raster_eval = true;            // separable evaluation on raster scan lists
     int order = 0;                      // scan contraction: 0 Gram matrix, 1 beam order, 2 probe order
     DevBuf ray, rax;                    // its phase tables
+    bool ray_scans = false;             // ... hold the phases of the scans in scans_d
     DevBuf aw1[6], aw2[6];              // per-target / per-parent weights (reconstruction adjoint)
     bool adj_tables = false;
     DevBuf f8pmax, f8inv0, f8inv1, f8hmax, f8H, f8sA, f8sB;   // FP8 per-window scales
     DevBuf errflag;
+    int* flag_h = nullptr;              // pinned copy of the flag
     std::vector<int32_t> work_h;
     bool check_finite = false;          // scan outputs for NaN / Inf (bip_set_check_finite)
     DevBuf nf_count;
@@ -486,6 +488,7 @@ bip_status make_tables(bip_ctx* c, cudaStream_t s) {
     CUDA_TRY(c, upload(c->hcube, hc, s));
     CUDA_TRY(c, upload(c->shcube, shc, s));
     CUDA_TRY(c, ensure(c->errflag, 64, true, s));
+    if (!c->flag_h) CUDA_TRY(c, cudaMallocHost((void**)&c->flag_h, 64));
     c->tables = true;
     return BIP_OK;
 }
@@ -821,6 +824,7 @@ bip_status bip_destroy(bip_ctx* c) {
                      &c->hcube, &c->shcube, &c->cstash, &c->ccols, &c->xopA, &c->xopB, &c->xm32, &c->tcache,
                      &c->cr_ay, &c->cr_ax, &c->cr_cy, &c->cr_cx, &c->cr_T, &c->nf_count, &c->tw512, &c->cols2, &c->gpart};
     for (DevBuf* b : all) release(*b);
+    if (c->flag_h) cudaFreeHost(c->flag_h);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->side) cudaStreamDestroy(c->side);
@@ -959,6 +963,16 @@ void release_map_workspaces(bip_ctx* c, cudaStream_t s) {
                       &c->s1t, &c->psi, &c->ybuf, &c->xtc, &c->f8pmax, &c->f8inv0, &c->f8inv1, &c->f8sA,
                       &c->f8sB})
         release(*b);
+}
+
+// Waits for the stream and turns the kernels' give-up flag into a status.
+// The flag comes back through pinned memory: a pageable copy waits for the
+// stream and then once more for itself (9 us).
+bip_status check_flag(bip_ctx* c, cudaStream_t s) {
+    CUDA_TRY(c, cudaMemcpyAsync(c->flag_h, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(c, cudaStreamSynchronize(s));
+    if (*c->flag_h) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
+    return BIP_OK;
 }
 
 // One FP32 contraction of cgemm_f32.cu: its plan, the workspace of a split k
@@ -1615,6 +1629,7 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
         CUDA_TRY(c, ensure(c->scans_d, (size_t)P * 2 * sizeof(double), false, s));
         CUDA_TRY(c, cudaMemcpyAsync(c->scans_d.p, scans, (size_t)P * 2 * sizeof(double), cudaMemcpyHostToDevice, s));
         c->scans_cache.assign(scans, scans + 2 * P);
+        c->ray_scans = false;
     }
     float* partial = partial_out;
     // beam order: the map as |M c|^2 summed over the detector beams on the
@@ -1633,6 +1648,7 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
                      g.ny, g.nx, (float2*)c->illum.p};
         CUDA_TRY(c, bip_illum(ia, s));
     }
+    Raster raster;
     if (cube_out) {
         // the cube cleared
         CUDA_TRY(c, cudaMemsetAsync(cube_out, 0, (size_t)P * geo.n_det * sizeof(float), s));
@@ -1641,38 +1657,34 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
             CUDA_TRY(c, ensure(c->partial, (size_t)c->n_sites * P * sizeof(float), false, s));
             partial = (float*)c->partial.p;
         }
+        if (!beam && !probe && c->raster_eval) raster = detect_raster(scans, P);
         // scans outside a site's crop mask stay 0: the evaluation writes only
-        // the scan tiles that can meet the mask
-        CUDA_TRY(c, cudaMemsetAsync(partial, 0, (size_t)c->n_sites * P * sizeof(float), s));
+        // the scan tiles that can meet the mask (a raster's writes every scan)
+        if (!raster.ok) CUDA_TRY(c, cudaMemsetAsync(partial, 0, (size_t)c->n_sites * P * sizeof(float), s));
     }
 
     // raster scan lists take the separable evaluation: phase tables per scan
     // row and column, angles reduced in FP64
-    Raster raster;
     RasterArgs rargs{};
-    if (!cube_out && !beam && !probe && c->raster_eval) raster = detect_raster(scans, P);
     if (raster.ok) {
         const int rows = 2 * c->Ky + 1, cols = 4 * c->Kx + 1;
-        if (!same_scans) {
-            std::vector<float2> ay((size_t)raster.My * rows), ax((size_t)cols * raster.Mx);
-            for (int my = 0; my < raster.My; ++my) {
-                const double ry = scans[2 * (size_t)my * raster.Mx];
-                for (int iy = 0; iy < rows; ++iy)
-                    ay[(size_t)my * rows + iy] = turn_d((double)g.fy * (iy - 2 * c->Ky) * ry / g.ny);
-            }
-            for (int mx = 0; mx < raster.Mx; ++mx) {
-                const double rx = scans[2 * (size_t)mx + 1];
-                for (int j = 0; j < cols; ++j) ax[(size_t)j * raster.Mx + mx] = turn_d((double)g.fx * (j - 2 * c->Kx) * rx / g.nx);
-            }
-            CUDA_TRY(c, upload(c->ray, ay, s));
-            CUDA_TRY(c, upload(c->rax, ax, s));
+        if (!c->ray_scans) {
+            if (capturing(s))
+                return fail(c, BIP_ERR_INVALID_ARG,
+                            "a captured map must repeat the arguments of the capture-safe warm-up call");
+            CUDA_TRY(c, ensure(c->ray, (size_t)raster.My * rows * sizeof(float2), false, s));
+            CUDA_TRY(c, ensure(c->rax, (size_t)cols * raster.Mx * sizeof(float2), false, s));
+            CUDA_TRY(c, bip_raster_tables(RasterTableArgs{raster.My, raster.Mx, c->Ky, c->Kx, g.fy, g.fx, g.ny, g.nx,
+                                                          (const double*)c->scans_d.p, (float2*)c->ray.p,
+                                                          (float2*)c->rax.p}, s));
+            c->ray_scans = true;
         }
         rargs = RasterArgs{raster.My, raster.Mx, (const float2*)c->ray.p, (const float2*)c->rax.p, raster.exact ? 1 : 0};
     }
 
     // scan-tile bounding boxes (host)
     std::vector<double> bb((size_t)n_tiles * 4);
-    for (int t = 0; t < n_tiles; ++t) {
+    for (int t = 0; t < n_tiles && !raster.ok; ++t) {
         double y0 = INFINITY, y1 = -INFINITY, x0 = INFINITY, x1 = -INFINITY;
         for (int p = t * tile; p < std::min(P, (t + 1) * tile); ++p) {
             y0 = std::min(y0, scans[2 * p]);
@@ -1730,7 +1742,8 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
     // work lists (site in batch, scan tile) for all batches, uploaded once
     // (kept across calls of a capture-safe context while scans, sites and
     // batching are unchanged)
-    const uint64_t work_key = (c->sig1 * 1000003ull) ^ ((uint64_t)SB << 32) ^ (uint64_t)P;
+    // -- none for a raster, whose evaluation takes every scan of a site at once
+    const uint64_t work_key = ((c->sig1 * 1000003ull) ^ ((uint64_t)SB << 32) ^ (uint64_t)P) * 2 + (raster.ok ? 1 : 0);
     const bool same_work = same_scans && c->work_key == work_key;
     std::vector<int32_t>& work = c->work_h;
     std::vector<int>& batch_off = c->batch_off_cache;
@@ -1741,7 +1754,7 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
         batch_off.push_back((int)work.size() / 2);
         for (int bs = 0; bs < bt.second; ++bs) {
             const SiteDev& sd = c->sites[c->batch_order[bt.first + bs]];
-            for (int t = 0; t < n_tiles; ++t)
+            for (int t = 0; t < n_tiles && !raster.ok; ++t)
                 if (box_meets_crop(bb[4 * t], bb[4 * t + 1], bb[4 * t + 2], bb[4 * t + 3], sd.ty, sd.tx, g)) {
                     work.push_back(bs);
                     work.push_back(t);
@@ -2198,17 +2211,16 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
         d.partial = partial;
         TIMED(c, BIP_STAGE_QUADFORM, s, bip_raster_eval(d, rargs, s));
     }
-    if (!c->capture_safe) {
-        int flag = 0;
-        CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(c, cudaStreamSynchronize(s));
-        if (flag) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
-    }
+    // the site sum goes out before the wait for the flag
     if (map_out && !cube_out) {
         CUDA_TRY(c, ensure(c->rsum, bip_reduce_scratch_bytes(c->n_sites, P), false, s));
         const double* occ = c->occ_n == c->n_sites ? (const double*)c->occ_d.p : nullptr;
         TIMED(c, BIP_STAGE_REDUCE, s, bip_reduce_sites(partial, c->n_sites, P, c->rsum.p, map_out, s, occ));
         if (c->n_sites > 0) c->launches[BIP_STAGE_REDUCE]++;   // two kernels: chunks, then their sum
+    }
+    if (!c->capture_safe) {
+        const bip_status st = check_flag(c, s);
+        if (st != BIP_OK) return st;
     }
     return BIP_OK;
 }
@@ -2591,10 +2603,8 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
         }
     }
     if (!c->capture_safe) {
-        int flag = 0;
-        CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(c, cudaStreamSynchronize(s));
-        if (flag) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
+        const bip_status st = check_flag(c, s);
+        if (st != BIP_OK) return st;
     }
     return BIP_OK;
 }
@@ -2714,13 +2724,13 @@ bip_status bip_debug_cgemm(bip_ctx* c, int32_t M, int32_t N, int32_t K, int32_t 
     p.B = CGemmOperand{(const float2*)B, sB[0], sB[1], sB[2], K, blocks, sB[3], 0, 0};
     p.conjA = flags & 1; p.conjB = flags >> 1 & 1; p.tri = flags >> 2 & 1;
     p.dk = w;
-    p.C = (float2*)C; p.scm = N; p.scb = (int64_t)M * N;
+    p.C = (float2*)C; p.scm = N; p.scn = 1; p.scb = (int64_t)M * N;
+    if (flags & 8) {                    // C(m, n) stored [n][m]
+        p.scm = 1;
+        p.scn = M;
+    }
     CUDA_TRY(c, cgemm(c, p, s));
-    int flag = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(c, cudaStreamSynchronize(s));
-    if (flag) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
-    return BIP_OK;
+    return check_flag(c, s);
 }
 
 bip_status bip_set_cube_memory(bip_ctx* c, int64_t bytes) {
@@ -3300,10 +3310,8 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
         }
     }
     {
-        int flag = 0;
-        CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(c, cudaStreamSynchronize(s));
-        if (flag) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
+        const bip_status st = check_flag(c, s);
+        if (st != BIP_OK) return st;
     }
     if (d_V) {
         CUDA_TRY(c, cudaMemsetAsync(d_V, 0, (size_t)g.nz * g.ny * g.nx * sizeof(float), s));
@@ -3572,10 +3580,8 @@ bip_status bip_site_coupling(bip_ctx* c, const void* H, int32_t site, void* m_ou
                                       tmp + (size_t)ch * Bpad, ldc * sizeof(float2), geo.B * sizeof(float2),
                                       geo.n_det, cudaMemcpyDeviceToDevice, s));
     {
-        int flag = 0;
-        CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(c, cudaStreamSynchronize(s));
-        if (flag) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
+        const bip_status st = check_flag(c, s);
+        if (st != BIP_OK) return st;
     }
     return BIP_OK;
 }

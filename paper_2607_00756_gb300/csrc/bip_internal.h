@@ -363,6 +363,15 @@ struct RasterArgs {
     int exact;                      // every row's y and every column's x bit for bit the same
 };
 cudaError_t bip_raster_eval(const DiffArgs& a, const RasterArgs& r, cudaStream_t s);
+// its phase tables from the scan list, ay[my][2 Ky + 1] = exp(2 pi i fy (iy - 2 Ky) ry / ny) and
+// ax[4 Kx + 1][mx] = exp(2 pi i fx (j - 2 Kx) rx / nx), in FP64
+struct RasterTableArgs {
+    int My, Mx, Ky, Kx, fy, fx, ny, nx;
+    const double* scans;
+    float2* ay;
+    float2* ax;
+};
+cudaError_t bip_raster_tables(const RasterTableArgs& a, cudaStream_t s);
 
 // reduce.cu : map[rho] = FP64 Neumaier sum over sites of the partials
 // (already zero outside each site's crop mask), in a fixed order; scratch

@@ -21,8 +21,8 @@
 //               lattice rows and over them, start angles reduced to [0, 1)
 //               turns in FP64.
 //   raster_eval: scans on a raster: the polynomial factorises over the two
-//               axes, two small dense stages per site (tables of the phases
-//               per scan row and column, angles reduced in FP64 on the host).
+//               axes, two small dense stages per site (raster_table: the
+//               phases per scan row and column, angles reduced in FP64).
 #include "bip_device.cuh"
 #include "bip_internal.h"
 #include "fft_smem.cuh"
@@ -154,6 +154,31 @@ __global__ void __launch_bounds__(256) diff_eval_kernel(DiffArgs a) {
     }
 }
 
+// The phase tables of a raster, one entry per thread in FP64 (about 10^4
+// entries at 128 x 128 scans, whose sines took the host 0.4 ms before the
+// map's first launch).
+__global__ void __launch_bounds__(128) raster_table_kernel(RasterTableArgs a) {
+    const int rows = 2 * a.Ky + 1, cols = 4 * a.Kx + 1, n_y = a.My * rows;
+    int i = blockIdx.x * 128 + threadIdx.x;
+    double t;
+    float2* o;
+    if (i < n_y) {
+        const int my = i / rows, iy = i % rows;
+        t = (double)a.fy * (iy - 2 * a.Ky) * a.scans[2 * (size_t)my * a.Mx] / a.ny;
+        o = a.ay + i;
+    } else {
+        i -= n_y;
+        if (i >= cols * a.Mx) return;
+        const int j = i / a.Mx, mx = i % a.Mx;
+        t = (double)a.fx * (j - 2 * a.Kx) * a.scans[2 * mx + 1] / a.nx;
+        o = a.ax + i;
+    }
+    t -= floor(t);
+    double s, c;
+    sincospi(2.0 * t, &s, &c);
+    *o = make_float2((float)c, (float)s);
+}
+
 // Raster scans: block = (4 WR scan rows, site), four warps of WR rows each;
 // stage 1 Y[r][j] = sum_iy Ay[my][iy] G[iy][j] for the block's rows into
 // shared memory, stage 2 lane = CX adjacent scan columns, WR rows x CX
@@ -228,7 +253,7 @@ __global__ void __launch_bounds__(128) raster_eval_kernel(DiffArgs a, RasterArgs
                 const int n = (my0 + q0 + q) * r.Mx + mx;
                 const bool in = r.exact ? cy[q0 + q] && cx[mx]
                                         : in_crop(a.scans[2 * n], a.scans[2 * n + 1], st.ty, st.tx, a.ny, a.nx, a.fy, a.fx);
-                if (in) a.partial[(size_t)site * a.P + n] = a.scale * acc[q][k];
+                a.partial[(size_t)site * a.P + n] = in ? a.scale * acc[q][k] : 0.f;
             }
         }
     }
@@ -266,6 +291,13 @@ cudaError_t bip_raster_eval(const DiffArgs& a, const RasterArgs& raster, cudaStr
     if (r.Mx > kRasterFlags) r.exact = 0;
     if ((int64_t)((r.My + 63) / 64) * a.n_sites >= 2 * 152) return launch_raster<16, 4>(a, r, s);
     return r.Mx > 64 ? launch_raster<4, 4>(a, r, s) : launch_raster<4, 1>(a, r, s);
+}
+
+cudaError_t bip_raster_tables(const RasterTableArgs& a, cudaStream_t s) {
+    const int64_t n = (int64_t)a.My * (2 * a.Ky + 1) + (int64_t)(4 * a.Kx + 1) * a.Mx;
+    if (n < 1 || n > 0x7fffff00) return cudaErrorInvalidValue;
+    raster_table_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t bip_diff_bin(const DiffArgs& a, cudaStream_t s) {
