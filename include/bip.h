@@ -524,7 +524,7 @@ bip_status bip_debug_allocs(int64_t* live, int64_t* made);
  *   C[z][m][n] = sum_kb sum_k opA(A(z, m, kb, k) w[k]) opB(B(z, kb, k, n)),
  * kb < blocks, k < K; op = conj with flag 1 (A) or 2 (B); flag 4: only the
  * tiles that reach the diagonal or lie right of it (the rest of C is left as
- * it is).  sA, sB: element strides of a row (m or n), of k, of the batch and
+ * it is); flag 8: C is written [batch][N][M].  sA, sB: element strides of a row (m or n), of k, of the batch and
  * of a block of k; of each operand's first two one is 1.  w (float32 [K],
  * nullable): with blocks = 1 only.  A, B, C complex64 device, C [batch][M][N].
  * BIP_ERR_INVALID_ARG for a null pointer, a size below 1 or such strides. */

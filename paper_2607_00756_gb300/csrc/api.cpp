@@ -996,25 +996,25 @@ cudaError_t cgemm(bip_ctx* c, CGemmF32 p, cudaStream_t s) {
 // (rows d), B [n_rows][K] the aperture side (rows (ch, b)), written transposed
 // as Mt[b][ch Dp + d] for the Gram step (ep_B = Bpad).
 CGemmF32 coupling_f32(int n_det, int n_rows, int K, const void* A, int64_t sA, const void* B, int64_t sB, void* C,
-                      int64_t ldc, int64_t sC, int Bpad, int Dp, int nb) {
+                      int64_t ldc, int64_t sC, int Bpad, int n_beams, int Dp, int nb) {
     CGemmF32 p{};
     p.M = n_det; p.N = n_rows; p.batch = nb;
     p.A = CGemmOperand{(const float2*)A, K, 1, sA, K, 1, 0, 0, 0};
     p.B = CGemmOperand{(const float2*)B, K, 1, sB, K, 1, 0, 0, 0};
     p.C = (float2*)C; p.scn = ldc; p.scb = sC;
-    p.ep_B = Bpad; p.ep_Dp = Dp;
+    p.ep_B = Bpad; p.ep_n = n_beams; p.ep_Dp = Dp;
     return p;
 }
 
 // The Gram matrix in FP32, Q = conj(Mt) Mt^T over K = (ch, d).  tri: only its
 // upper triangle (what the scan polynomial reads).
-CGemmF32 gram_f32(int Bpad, int64_t ldm, const void* Mt, int64_t sM, void* Q, int64_t sQ, bool tri, int nb) {
+CGemmF32 gram_f32(int B, int Bpad, int64_t ldm, const void* Mt, int64_t sM, void* Q, int64_t sQ, bool tri, int nb) {
     CGemmF32 p{};
-    p.M = Bpad; p.N = Bpad; p.batch = nb;
+    p.M = B; p.N = B; p.batch = nb;
     p.A = CGemmOperand{(const float2*)Mt, ldm, 1, sM, (int)ldm, 1, 0, 0, 0};
     p.B = p.A;
     p.conjA = 1;
-    p.C = (float2*)Q; p.scm = Bpad; p.scb = sQ;
+    p.C = (float2*)Q; p.scm = Bpad; p.scn = 1; p.scb = sQ;
     p.tri = tri ? 1 : 0;
     return p;
 }
@@ -2145,7 +2145,7 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
             // coupling M = S2^T diag(H) S1, stored transposed for the Gram step
             TIMED(c, BIP_STAGE_COUPLING, s,
                   cgemm(c, coupling_f32(geo.n_det, (int)rowsB, K, c->opA32.p, (int64_t)perA, c->opB32.p, (int64_t)perB,
-                                        c->mt32.p, (int64_t)nch * Dpad, (int64_t)perMt, Bpad, Dpad, nb), s));
+                                        c->mt32.p, (int64_t)nch * Dpad, (int64_t)perMt, Bpad, geo.B, Dpad, nb), s));
             if (sepq) {
                 CubeRasterArgs r = cra;
                 r.n_sites = nb;
@@ -2165,7 +2165,7 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
             }
             // Gram Q = sum_n M^(n)H M^(n), upper triangle
             TIMED(c, BIP_STAGE_GRAM, s,
-                  cgemm(c, gram_f32(Bpad, (int64_t)nch * Dpad, c->mt32.p, (int64_t)perMt, c->q32.p, (int64_t)perQ, true,
+                  cgemm(c, gram_f32(geo.B, Bpad, (int64_t)nch * Dpad, c->mt32.p, (int64_t)perMt, c->q32.p, (int64_t)perQ, true,
                                     nb), s));
         }
         // I_tau(rho) = f_y f_x c^H Q c as a trigonometric polynomial over
@@ -2579,7 +2579,7 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
             } else {
                 TIMED(c, BIP_STAGE_COUPLING, s,
                       cgemm(c, coupling_f32(nd, (int)rowsB, K, c->xopA.p, (int64_t)perA, c->xopB.p, (int64_t)perB,
-                                            c->xm32.p, (int64_t)nch * Dpb, (int64_t)perMt, Bpad, Dpb, nb), s));
+                                            c->xm32.p, (int64_t)nch * Dpb, (int64_t)perMt, Bpad, geo.B, Dpb, nb), s));
                 if (sep) {
                     CubeRasterArgs r = cra;
                     r.n_sites = nb;
@@ -3156,7 +3156,7 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
             CUDA_TRY(c, bip_tc_gemm(A, s));
         } else {
             CUDA_TRY(c, cgemm(c, coupling_f32(geo.n_det, nch * Bpad, K, c->opA32.p, (int64_t)perA, c->opB32.p,
-                                              (int64_t)perB, c->mt32.p, (int64_t)ldm, (int64_t)perMt, Bpad, Dpad, nb), s));
+                                              (int64_t)perB, c->mt32.p, (int64_t)ldm, (int64_t)perMt, Bpad, geo.B, Dpad, nb), s));
         }
         // R_tau = f o_tau sum_{rho in crop} g c c^H
         CUDA_TRY(c, bip_grad_crop_weights(gab, nb, ids, (float*)c->g_w.p, s));
@@ -3166,23 +3166,24 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
         r.dk = (const float*)c->g_w.p; r.sdb = P;
         r.B = r.A;
         r.conjB = 1;
-        r.C = (float2*)c->g_R.p; r.scm = Bpad; r.scb = (int64_t)perQ;
+        r.C = (float2*)c->g_R.p; r.scm = Bpad; r.scn = 1; r.scb = (int64_t)perQ;
         CUDA_TRY(c, cgemm(c, r, s));
         if (d_aberr) {
             // Q = sum_n M_n^H M_n, then D_b += (Q R)_bb
-            CUDA_TRY(c, cgemm(c, gram_f32(Bpad, (int64_t)ldm, c->mt32.p, (int64_t)perMt, c->q32.p, (int64_t)perQ, false,
+            CUDA_TRY(c, cgemm(c, gram_f32(geo.B, Bpad, (int64_t)ldm, c->mt32.p, (int64_t)perMt, c->q32.p, (int64_t)perQ, false,
                                           nb), s));
             CUDA_TRY(c, bip_grad_aberr(B, Bpad, nb, (const float2*)c->q32.p, (int64_t)perQ, (const float2*)c->g_R.p,
                                        (int64_t)perQ, (double2*)c->g_D.p, (double2*)c->g_Dsum.p, s));
         }
         if (d_H || d_V) {
             // Mbar_n = M_n R, kept as GMt = conj(R) Mt (R Hermitian)
+            // (the rows (n, d) as the contraction's rows, the beams as its columns)
             CGemmF32 m{};
-            m.M = B; m.N = (int)ldm; m.batch = nb;
-            m.A = CGemmOperand{(const float2*)c->g_R.p, Bpad, 1, (int64_t)perQ, B, 1, 0, 0, 0};
-            m.conjA = 1;
-            m.B = CGemmOperand{(const float2*)c->mt32.p, 1, (int64_t)ldm, (int64_t)perMt, B, 1, 0, 0, 0};
-            m.C = (float2*)c->g_gmt.p; m.scm = (int64_t)ldm; m.scb = (int64_t)perMt;
+            m.M = (int)ldm; m.N = B; m.batch = nb;
+            m.A = CGemmOperand{(const float2*)c->mt32.p, 1, (int64_t)ldm, (int64_t)perMt, B, 1, 0, 0, 0};
+            m.B = CGemmOperand{(const float2*)c->g_R.p, Bpad, 1, (int64_t)perQ, B, 1, 0, 0, 0};
+            m.conjB = 1;
+            m.C = (float2*)c->g_gmt.p; m.scm = 1; m.scn = (int64_t)ldm; m.scb = (int64_t)perMt;
             CUDA_TRY(c, cgemm(c, m, s));
             // T_n(b, r) = sum_d Mbar_n(d, b) conj S2_d(r)
             if (tcg) {
@@ -3218,12 +3219,12 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
                     CUDA_TRY(c, bip_tc_gemm(t, s));
                 } else {
                     CGemmF32 t{};
-                    t.M = B; t.N = K; t.batch = nb;
-                    t.A = CGemmOperand{(const float2*)c->g_gmt.p + (size_t)n * Dpad, (int64_t)ldm, 1, (int64_t)perMt,
+                    t.M = K; t.N = B; t.batch = nb;
+                    t.A = CGemmOperand{(const float2*)c->opA32.p, 1, K, (int64_t)perA, geo.n_det, 1, 0, 0, 0};
+                    t.conjA = 1;
+                    t.B = CGemmOperand{(const float2*)c->g_gmt.p + (size_t)n * Dpad, (int64_t)ldm, 1, (int64_t)perMt,
                                        geo.n_det, 1, 0, 0, 0};
-                    t.B = CGemmOperand{(const float2*)c->opA32.p, 1, K, (int64_t)perA, geo.n_det, 1, 0, 0, 0};
-                    t.conjB = 1;
-                    t.C = (float2*)c->g_T.p + (size_t)n * Bpad * K; t.scm = K; t.scb = (int64_t)perT;
+                    t.C = (float2*)c->g_T.p + (size_t)n * Bpad * K; t.scm = 1; t.scn = K; t.scb = (int64_t)perT;
                     CUDA_TRY(c, cgemm(c, t, s));
                 }
             }
@@ -3271,7 +3272,7 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
                 u.A = CGemmOperand{(const float2*)c->g_gmt.p, 1, (int64_t)ldm, (int64_t)perMt, B, nch, Dpad, 0, 0};
                 u.B = CGemmOperand{(const float2*)c->opB32.p, 1, K, (int64_t)perB, B, nch, (int64_t)Bpad * K, 0, 0};
                 u.conjB = 1;
-                u.C = (float2*)c->g_s2bar.p; u.scm = K; u.scb = (int64_t)perS2bar;
+                u.C = (float2*)c->g_s2bar.p; u.scm = K; u.scn = 1; u.scb = (int64_t)perS2bar;
                 CUDA_TRY(c, cgemm(c, u, s));
             }
             // back through the reconstructions into the window adjoints
@@ -3570,8 +3571,9 @@ bip_status bip_site_coupling(bip_ctx* c, const void* H, int32_t site, void* m_ou
         }
         TIMED(c, BIP_STAGE_COUPLING, s, bip_tc_gemm(A, s));
     } else {
-        CGemmF32 A = coupling_f32(geo.n_det, (int)ldc, K, opA.p, (int64_t)perA, opB.p, (int64_t)perB, tmp, 0, 0, 0, 0, 1);
+        CGemmF32 A = coupling_f32(geo.n_det, (int)ldc, K, opA.p, (int64_t)perA, opB.p, (int64_t)perB, tmp, 0, 0, 0, 0, 0, 1);
         A.scm = (int64_t)ldc;
+        A.scn = 1;
         TIMED(c, BIP_STAGE_COUPLING, s, cgemm(c, A, s));
     }
     // [n_det][(ch, b)] -> m_out[ch][n_det][B]

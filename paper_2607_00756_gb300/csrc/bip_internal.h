@@ -309,17 +309,17 @@ struct CGemmF32 {
     CGemmOperand A, B;
     int conjA, conjB;
     const float* dk; int64_t sdb;   // optional real scale of each k (null: 1), with one k block only
-    // C(m, n) at C[z scb + m scm + n], or with ep_B > 0 (n = (ch, b)) at
-    // C[z scb + b scn + ch ep_Dp + m]
+    // C(m, n) at C[z scb + m scm + n scn], or with ep_B > 0 (n = (ch, b) = ch
+    // ep_B + b, of which b < ep_n are computed) at C[z scb + b scn + ch ep_Dp + m]
     float2* C; int64_t scm, scn, scb;
-    int ep_B, ep_Dp;
+    int ep_B, ep_n, ep_Dp;
     int tri;                        // only the column tiles that reach the diagonal or lie right of it
     int plan_batch;                 // batch size the k split is chosen for (0: batch)
     float2* part;                   // workspace of a split k range
     int* err;
     uint64_t wait_ns;
     // (plan)
-    int nt, n_tiles, tiles, steps, ksplit, units, vecC;
+    int nt, n_tiles, ch_tiles, tiles, steps, ksplit, units, vecC;
 };
 // fills the plan; *part_elems: float2 elements `part` must hold (0: none)
 cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems);

@@ -54,6 +54,8 @@ constexpr int kThreads = 32 * (kIssuer + 4);
 constexpr int kRegsLaunch = 96, kRegsCut = 64, kRegsAdd = 152, kRegsIssue = 40;
 static_assert(32 * (kCut * kRegsCut + kAdd * kRegsAdd + 4 * kRegsIssue) <= kThreads * kRegsLaunch,
               "the split draws on the registers of the launch");
+static_assert(kRegsCut <= kRegsLaunch && kRegsIssue <= kRegsLaunch && kRegsAdd >= kRegsLaunch,
+              "setmaxnreg.dec gives registers back, .inc takes some");
 constexpr int kStep = 16;                        // complex k per chunk
 constexpr int kALevel = 128 * 64, kBLevel = 256 * 64;   // bytes of one term of a stage
 constexpr int kStage = 3 * (kALevel + kBLevel);
@@ -85,7 +87,7 @@ __device__ __forceinline__ bool wait_long(uint64_t* b, uint32_t parity, volatile
 }
 
 struct Unit {
-    int z, m0, n0, ks;
+    int z, m0, n0, n1, ks;                       // columns [n0, n1)
     int s0, s1;                                  // steps [s0, s1)
 };
 
@@ -113,7 +115,14 @@ __device__ __forceinline__ bool unit_of(const CGemmF32& p, int i, Unit& u) {
         u.m0 = r / p.n_tiles * 128;
         r %= p.n_tiles;
     }
-    u.n0 = r * p.nt;
+    if (p.ep_B > 0) {
+        // the tiles of a channel's ep_n columns
+        u.n0 = r / p.ch_tiles * p.ep_B + r % p.ch_tiles * p.nt;
+        u.n1 = min(u.n0 + p.nt, r / p.ch_tiles * p.ep_B + p.ep_n);
+    } else {
+        u.n0 = r * p.nt;
+        u.n1 = min(u.n0 + p.nt, p.N);
+    }
     u.s0 = (int)((int64_t)p.steps * u.ks / p.ksplit);
     u.s1 = (int)((int64_t)p.steps * (u.ks + 1) / p.ksplit);
     return true;
@@ -284,7 +293,7 @@ __device__ __forceinline__ int64_t out_at(const CGemmF32& p, int z, int m, int n
     int64_t o = (int64_t)z * p.scb;
     if (p.ep_B > 0)                              // the coupling as the Gram operand: n = (ch, b), m = d
         return o + (int64_t)(n % p.ep_B) * p.scn + (int64_t)(n / p.ep_B) * p.ep_Dp + m;
-    return o + (int64_t)m * p.scm + n;
+    return o + (int64_t)m * p.scm + (int64_t)n * p.scn;
 }
 
 template <bool AKC, bool BKC>
@@ -404,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
         float2 va[8], vb[8];
         auto load = [&]() {
             load8<AKC>(va, p.A, p.A.p + (int64_t)u.z * p.A.sb, u.m0, p.M, sla, st);
-            load8<BKC>(vb, p.B, p.B.p + (int64_t)u.z * p.B.sb, u.n0, p.N, slb, st);
+            load8<BKC>(vb, p.B, p.B.p + (int64_t)u.z * p.B.sb, u.n0, u.n1, slb, st);
             if (p.dk) {
                 const float* w = p.dk + (int64_t)u.z * p.sdb;
 #pragma unroll
@@ -484,7 +493,7 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
             }
             const int m = u.m0 + (warp & 3) * 32 + lane;
             if (!ok || m >= p.M) continue;
-            const int n0 = u.n0 + c0, n1 = min(p.nt, p.N - u.n0) - c0;   // this warp's columns
+            const int n0 = u.n0 + c0, n1 = u.n1 - n0;          // this warp's columns
             float2* o;
             bool vec = false;
             if (p.ksplit > 1) {
@@ -499,7 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
                 for (int j = 0; j < 8; ++j) {
                     const int n = 16 * g + 2 * j;
                     const float2 re = unpack2(acc[0][g][j]), im = unpack2(acc[1][g][j]);
-                    if (p.ep_B > 0 && p.ksplit == 1) {
+                    if ((p.ep_B > 0 || p.scn != 1) && p.ksplit == 1) {
                         if (n < n1) p.C[out_at(p, u.z, m, n0 + n)] = make_float2(re.x, im.x);
                         if (n + 1 < n1) p.C[out_at(p, u.z, m, n0 + n + 1)] = make_float2(re.y, im.y);
                     } else if (vec && n + 1 < n1) {
@@ -529,6 +538,7 @@ __global__ void __launch_bounds__(256) cgemm_sum_kernel(const CGemmF32 p) {
     const int64_t zm = i / p.N;
     const int m = (int)(zm % p.M), z = (int)(zm / p.M);
     if (p.tri && n < m / 128 * 128 / p.nt * p.nt) return;     // tiles left of the diagonal's are not computed
+    if (p.ep_B > 0 && n % p.ep_B >= p.ep_n) return;
     float2 v = p.part[i];
     for (int k = 1; k < p.ksplit; ++k) {
         const float2 w = p.part[(int64_t)k * n_el + i];
@@ -563,7 +573,11 @@ bool aligned2(const void* q, int64_t a, int64_t b, int64_t c) {
 
 // Tile widths, the k split and the workspace (float2 elements of `part`).
 // The column tile is the narrowest multiple of 8 that keeps the tile count of
-// 128-wide ones (no work for padding columns beyond 7).  The split: the parts
+// 128-wide ones, and the coupling's columns are tiled channel by channel, so
+// that no padding columns beyond 7 are computed (45 beams padded to 128 rows
+// per channel: 3 tiles of 48; 4 sites' coupling and Gram 111 us in whole
+// tiles, 74 us in these).  Callers put the side with few rows on the columns for the same
+// reason: its rows would be padded to 128.  The split: the parts
 // that minimise rounds x (chunks per part + the pipeline's fill, about three
 // chunks), plus the parts' way through memory at about 2.5 KB per clock.  It
 // is chosen for plan_batch entries, so that a site's sums do not depend on
@@ -581,10 +595,13 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
     }
     if (p.A.kvalid != p.B.kvalid || p.A.nper != p.B.nper) return cudaErrorInvalidValue;
     if (p.dk && p.A.nper != 1) return cudaErrorInvalidValue;
-    p.vecC = aligned2(p.C, p.scm, p.scb, 0) ? 1 : 0;
-    p.n_tiles = (p.N + 127) / 128;
-    p.nt = ((p.N + p.n_tiles - 1) / p.n_tiles + 7) / 8 * 8;
-    p.n_tiles = (p.N + p.nt - 1) / p.nt;
+    p.vecC = p.scn == 1 && aligned2(p.C, p.scm, p.scb, 0) ? 1 : 0;
+    if (p.ep_B > 0 && (p.ep_n < 1 || p.ep_n > p.ep_B || p.N % p.ep_B)) return cudaErrorInvalidValue;
+    const int cols = p.ep_B > 0 ? p.ep_n : p.N;                // of a channel, or all
+    p.ch_tiles = (cols + 127) / 128;
+    p.nt = ((cols + p.ch_tiles - 1) / p.ch_tiles + 7) / 8 * 8;
+    p.ch_tiles = (cols + p.nt - 1) / p.nt;
+    p.n_tiles = p.ch_tiles * (p.ep_B > 0 ? p.N / p.ep_B : 1);
     const int m_tiles = (p.M + 127) / 128;
     p.tiles = 0;
     for (int mt = 0; mt < m_tiles; ++mt) p.tiles += p.n_tiles - (p.tri ? mt * 128 / p.nt : 0);

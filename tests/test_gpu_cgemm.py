@@ -72,6 +72,19 @@ def test_against_complex128(env, M, N, K, blocks, batch, layout, pad, flags):
     assert torch.all((C - want).abs() <= bound(blocks * K) * size)
 
 
+@pytest.mark.parametrize("M,N,K,blocks,batch,layout,pad", CASES[3:9])
+def test_transposed_output(env, M, N, K, blocks, batch, layout, pad):
+    capi, ctx = env
+    rng = torch.Generator("cuda").manual_seed(M + N + K)
+    A, sA, _ = operand(rng, M, K, blocks, batch, layout[0], pad)
+    B, sB, _ = operand(rng, N, K, blocks, batch, layout[1], pad)
+    C = torch.full((batch, M, N), float("nan"), dtype=torch.complex64, device="cuda")
+    T = torch.full((batch, N, M), float("nan"), dtype=torch.complex64, device="cuda")
+    capi.bip_debug_cgemm(ctx, M, N, K, blocks, batch, A, sA, B, sB, 0, None, C)
+    capi.bip_debug_cgemm(ctx, M, N, K, blocks, batch, A, sA, B, sB, 8, None, T)
+    assert torch.equal(torch.view_as_real(C), torch.view_as_real(T.transpose(1, 2).contiguous()))
+
+
 @pytest.mark.parametrize("M", [64, 128, 256, 384, 513])
 def test_upper_triangle(env, M):
     """Hermitian products: every column tile that reaches the diagonal or
