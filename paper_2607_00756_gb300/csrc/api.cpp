@@ -70,7 +70,7 @@ struct bip_ctx {
     DevBuf cols2;                       // S2's columns while both sweeps run at once (bip_build)
     cudaStream_t side = nullptr;        // bip_build: the stream S2's sweep runs on
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    DevBuf tw512;                       // nx = 512: the half-warp row pass's twiddles
+    DevBuf twhw;                        // the half-warp row pass's twiddles
 
     // map workspaces
     DevBuf scans_d, work_d, partial, gdiff, rsum, illum, cube_scratch, bin_of_d;
@@ -435,12 +435,15 @@ bip_status make_tables(bip_ctx* c, cudaStream_t s) {
         for (int v = 0; v < g.win; ++v) xt[(size_t)h * g.win + v] = turn((int)((int64_t)h * v % g.nx), g.nx, +1.0);
     CUDA_TRY(c, upload(c->twy, twy, s));
     CUDA_TRY(c, upload(c->twx, twx, s));
-    if (g.nx == 512) {
-        // twiddles of the half-warp row pass's second pass
-        std::vector<float2> t5(15 * 32);
-        for (int e = 1; e < 16; ++e)
-            for (int j = 0; j < 32; ++j) t5[(size_t)(e - 1) * 32 + j] = turn(e * j, 512, -1.0);
-        CUDA_TRY(c, upload(c->tw512, t5, s));
+    // twiddles of the half-warp row pass's second pass.  At 1024 points its
+    // roundings differ from the radix-8 pass's, and E4M3 codes move with them,
+    // so FP8 contexts keep that pass there.
+    if (g.nx == 256 || g.nx == 512 || (g.nx == 1024 && g.prec != BIP_PREC_FP8_TILE)) {
+        const int r1 = g.nx == 256 ? 16 : 32, r2 = g.nx / r1;
+        std::vector<float2> t2((size_t)(r2 - 1) * r1);
+        for (int e = 1; e < r2; ++e)
+            for (int j = 0; j < r1; ++j) t2[(size_t)(e - 1) * r1 + j] = turn(e * j, g.nx, -1.0);
+        CUDA_TRY(c, upload(c->twhw, t2, s));
     }
     CUDA_TRY(c, upload(c->ey, ey, s));
     CUDA_TRY(c, upload(c->ex, ex, s));
@@ -650,7 +653,7 @@ MsPlan plan_for(bip_ctx* c, int ncol, const DevBuf& shift) {
     p.py = (const float2*)c->py.p;
     p.px = (const float2*)c->px.p;
     p.shift = (const int2*)shift.p;
-    p.tw512 = c->cfg.nx == 512 ? (const float2*)c->tw512.p : nullptr;
+    p.twhw = (const float2*)c->twhw.p;
     return p;
 }
 
@@ -822,7 +825,7 @@ bip_status bip_destroy(bip_ctx* c) {
                      &c->ray, &c->rax, &c->g_tA, &c->g_tB, &c->g_sA2, &c->g_sB2, &c->cubeA, &c->cubeB,
                      &c->cube_work, &c->cube_mask, &c->s1t, &c->psi, &c->ybuf, &c->cube_grp, &c->cube_wmap, &c->mpart,
                      &c->hcube, &c->shcube, &c->cstash, &c->ccols, &c->xopA, &c->xopB, &c->xm32, &c->tcache,
-                     &c->cr_ay, &c->cr_ax, &c->cr_cy, &c->cr_cx, &c->cr_T, &c->nf_count, &c->tw512, &c->cols2, &c->gpart};
+                     &c->cr_ay, &c->cr_ax, &c->cr_cy, &c->cr_cx, &c->cr_T, &c->nf_count, &c->twhw, &c->cols2, &c->gpart};
     for (DevBuf* b : all) release(*b);
     if (c->flag_h) cudaFreeHost(c->flag_h);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);

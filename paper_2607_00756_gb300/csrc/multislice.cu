@@ -12,9 +12,9 @@
 // unnormalised forward/inverse FFT pair.
 //
 // Grid lengths: powers of two 64..1024, and 3 M (192, 384, 768) through
-// the radix-3 layer of the register FFT (fft_reg3).  Rows of 512 points
-// (the paper-scale grids) take a two-pass form on half-warps when the plan
-// carries its twiddle table (row_pass_hw512_kernel).
+// the radix-3 layer of the register FFT (fft_reg3).  Rows of 256, 512 and
+// 1024 points take a two-pass form on half-warps or warps when the plan
+// carries its twiddle table (row_pass_hw_kernel).
 //
 // One step of a column is two passes over global memory:
 //   row pass    [inverse FFT along x] [T_pre] [stash, save] [T_post] [FFT along x]
@@ -179,25 +179,34 @@ __global__ void __launch_bounds__(kThreads) row_pass_kernel(MsPlan plan, MsRowAr
 }
 
 // ---------------------------------------------------------------------------
-// Rows of 512 points on half-warps.  512 = 32 x 16, so a transform is two
-// register passes with one exchange between them: pass 1 a DFT-32 per
-// thread over x[t + 16 m] (m = 0..31), pass 2 two DFT-16 per thread, each
-// after a twiddle by exp(-+2 pi i e j / 512).  Sixteen threads hold a row in
-// the cyclic layout x = t + 16 m in both domains, so the row never leaves
-// its half-warp: the exchange needs __syncwarp only, and against the
-// radix-8 form above it moves every value through shared memory once per
-// transform instead of twice and reads half the twiddles.  A block of 256
-// threads takes 16 parent columns at one y.
+// Rows of 256, 512 and 1024 points on half-warps (1024: warps).  N = R1 x R2,
+// so a transform is two register passes with one exchange between them: pass
+// 1 a DFT-R1 per thread over x[t + NT m] (m < R1), pass 2 NB DFT-R2 per thread,
+// each after a twiddle by exp(-+2 pi i e j / N).  NT threads hold a row in the
+// cyclic layout x = t + NT m in both domains, so the row never leaves its
+// (half-)warp: the exchange needs __syncwarp only, and against the radix-8
+// form above it moves every value through shared memory once per transform
+// instead of twice and reads half the twiddles.  A block takes RPB parent
+// columns at one y.
 //
 // Local DFTs of length L = 4 B (B = 8 or 4), natural order in and out:
 // with n = n1 + 4 n2 and k = B k1 + k2, a DFT-B over n2 for each n1, the
 // twiddle W_L^(n1 k2), then a DFT-4 over n1 for each k2.
-namespace hw512 {
+namespace hw {
 
-constexpr int N = 512, NT = 16, NV = 32;
-constexpr int RPB = kThreads / NT;                 // rows (parent columns) per block
-constexpr int ROWBUF = N + N / 32;                 // exchange entries per row: one pad per 32
-constexpr int NTW = 15 * 32;                       // pass-2 twiddles [e - 1][j]
+template <int LEN>
+struct Row {
+    static constexpr int N = LEN;
+    static constexpr int R1 = LEN == 256 ? 16 : 32, R2 = LEN / R1;
+    static constexpr int NT = LEN / R1, NV = R1;         // threads and values per thread of a row
+    static constexpr int NB = R1 / NT;                   // pass-2 butterflies per thread
+    static constexpr int THREADS = LEN == 256 ? 128 : 256;
+    static constexpr int RPB = THREADS / NT;
+    static constexpr int BUF = N + N / R1;               // exchange entries per row: one pad per R1
+    static constexpr int NTW = (R2 - 1) * R1;            // pass-2 twiddles [e - 1][j]
+    static constexpr int MINB = LEN == 256 ? 8 : 2;      // blocks per SM the registers are set for
+    static constexpr size_t SMEM = ((size_t)RPB * BUF + NTW + 2 * N) * sizeof(float2);
+};
 
 // exp(-2 pi i m / 32)
 __constant__ float2 kW32[32] = {
@@ -250,7 +259,7 @@ __device__ __forceinline__ void dft16(float2 (&u)[16]) {
 }
 
 template <bool INV>
-__device__ __forceinline__ void dft32(float2 (&v)[NV]) {
+__device__ __forceinline__ void dft32(float2 (&v)[32]) {
     float2 b[4][8];
 #pragma unroll
     for (int n1 = 0; n1 < 4; ++n1) {
@@ -268,39 +277,46 @@ __device__ __forceinline__ void dft32(float2 (&v)[NV]) {
     }
 }
 
-// One length-512 transform of the row held by this half-warp (thread t:
-// v[m] = x[t + 16 m] on entry, X[t + 16 m] on exit; unnormalised inverse).
-// buf: this row's exchange buffer (entry i at i + i / 32); tw2: the pass-2
-// twiddles exp(-2 pi i e j / 512) at (e - 1) 32 + j.  Every lane of the warp
-// calls it (the warp's two rows together).
-template <bool INV>
-__device__ __forceinline__ void fft512(float2 (&v)[NV], float2* buf, int t, const float2* tw2) {
-    dft32<INV>(v);
-    // pass-1 output r of butterfly t is y[32 t + r]
+template <bool INV, int R>
+__device__ __forceinline__ void dft(float2 (&v)[R]) {
+    if constexpr (R == 32) dft32<INV>(v);
+    else dft16<INV>(v);
+}
+
+// One length-N transform of the row held by NT lanes (thread t: v[m] =
+// x[t + NT m] on entry, X[t + NT m] on exit; unnormalised inverse).  buf: this
+// row's exchange buffer (entry i at i + i / R1); tw2: the pass-2 twiddles
+// exp(-2 pi i e j / N) at (e - 1) R1 + j.  Every lane of the warp calls it (the
+// warp's rows together).
+template <class H, bool INV>
+__device__ __forceinline__ void fft_row(float2 (&v)[H::NV], float2* buf, int t, const float2* tw2) {
+    constexpr int R1 = H::R1, R2 = H::R2;
+    dft<INV, R1>(v);
+    // pass-1 output r of butterfly t is y[R1 t + r]
 #pragma unroll
-    for (int r = 0; r < 32; ++r) buf[33 * t + r] = v[r];
+    for (int r = 0; r < R1; ++r) buf[(R1 + 1) * t + r] = v[r];
     __syncwarp();
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int j = t + 16 * h;                  // pass-2 butterfly: y[j + 32 e], e < 16
-        float2 u[16];
+    for (int h = 0; h < H::NB; ++h) {
+        const int j = t + H::NT * h;               // pass-2 butterfly: y[j + R1 e], e < R2
+        float2 u[R2];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) u[e] = buf[j + 33 * e];
+        for (int e = 0; e < R2; ++e) u[e] = buf[j + (R1 + 1) * e];
 #pragma unroll
-        for (int e = 1; e < 16; ++e) {
-            float2 w = tw2[(e - 1) * 32 + j];
+        for (int e = 1; e < R2; ++e) {
+            float2 w = tw2[(e - 1) * R1 + j];
             if (INV) w.y = -w.y;
             u[e] = c_mul(u[e], w);
         }
-        dft16<INV>(u);
-        // output r is X[j + 32 r] = X[t + 16 (2 r + h)]
+        dft<INV, R2>(u);
+        // output r is X[j + R1 r] = X[t + NT (NB r + h)]
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[2 * r + h] = u[r];
+        for (int r = 0; r < R2; ++r) v[H::NB * r + h] = u[r];
     }
     __syncwarp();                                  // reads done before the buffer is reused
 }
 
-}  // namespace hw512
+}  // namespace hw
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
@@ -309,7 +325,7 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// The row pass of row_pass_kernel<512> on half-warp rows (same arguments,
+// The row pass of row_pass_kernel<N> on half-warp (warp) rows (same arguments,
 // same results up to rounding order), persistent over the grid rows: block
 // b keeps the column group b % groups and takes the rows y = b / groups,
 // + blocks / groups, ...  While a half-warp stores its row it already copies
@@ -317,14 +333,16 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // cp.async, and the block copies the next row's transmission into the
 // other of two T buffers, so the loads of one row overlap the work of the
 // previous one.
-__global__ void __launch_bounds__(kThreads, 2) row_pass_hw512_kernel(MsPlan plan, MsRowArgs a, int groups) {
-    using namespace hw512;
+template <int LEN>
+__global__ void __launch_bounds__(hw::Row<LEN>::THREADS, hw::Row<LEN>::MINB) row_pass_hw_kernel(MsPlan plan, MsRowArgs a, int groups) {
+    using H = hw::Row<LEN>;
+    constexpr int N = H::N, NT = H::NT, NV = H::NV, RPB = H::RPB;
     extern __shared__ float2 smem[];
     const int sub = threadIdx.x / NT;
     const int t = threadIdx.x % NT;
-    float2* buf = smem + sub * ROWBUF;
-    float2* tw2 = smem + RPB * ROWBUF;             // [15][32]
-    float2* tts = tw2 + NTW;                       // [2][512] transmission of the current / next y
+    float2* buf = smem + sub * H::BUF;
+    float2* tw2 = smem + RPB * H::BUF;             // [R2 - 1][R1]
+    float2* tts = tw2 + H::NTW;                    // [2][N] transmission of the current / next y
     const int cg = blockIdx.x % groups;
     const int ystep = gridDim.x / groups;          // the launch makes gridDim.x a multiple of groups
     const int c = cg * RPB + sub;
@@ -340,9 +358,11 @@ __global__ void __launch_bounds__(kThreads, 2) row_pass_hw512_kernel(MsPlan plan
         if (load) {
             const float2* src = gcol + (size_t)y * N;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) cp_async16(buf + 2 * (t + 16 * k), src + 2 * (t + 16 * k));
+            for (int k = 0; k < NV / 2; ++k) cp_async16(buf + 2 * (t + NT * k), src + 2 * (t + NT * k));
         }
-        if (table) cp_async16(tts + slot * N + 2 * threadIdx.x, a.t_slice + (size_t)y * N + 2 * threadIdx.x);
+        if (table)
+            for (int i = 2 * threadIdx.x; i < N; i += 2 * H::THREADS)
+                cp_async16(tts + slot * N + i, a.t_slice + (size_t)y * N + i);
         cp_async_commit();
     };
 
@@ -356,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_pass_hw512_kernel(MsPlan plan
         }
     };
 
-    for (int i = threadIdx.x; i < NTW; i += kThreads) tw2[i] = __ldg(&plan.tw512[i]);
+    for (int i = threadIdx.x; i < H::NTW; i += H::THREADS) tw2[i] = __ldg(&plan.twhw[i]);
     int y = blockIdx.x / groups;
     int slot = 0;
     int e0, e1;
@@ -364,11 +384,11 @@ __global__ void __launch_bounds__(kThreads, 2) row_pass_hw512_kernel(MsPlan plan
     if (y < plan.ny) prefetch(y, 0);
     for (; y < plan.ny; y += ystep, slot ^= 1) {
         float2* tt = tts + slot * N;
-        // the first 16 entries, one per lane, in flight during the inverse transform
+        // the first NT entries, one per lane, in flight during the inverse transform
         int4 ent = make_int4(0, 0, 0, 0);
         if (e0 + t < e1) ent = __ldg(&a.row_ent[e0 + t]);
         if (vsl && !a.t_slice) {
-            for (int i = threadIdx.x; i < N; i += kThreads) {
+            for (int i = threadIdx.x; i < N; i += H::THREADS) {
                 float sn, co;
                 sincosf(plan.sigma * __ldg(&vsl[(size_t)y * N + i]), &sn, &co);
                 tt[i] = make_float2(co, sn);
@@ -381,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_pass_hw512_kernel(MsPlan plan
         for (int m = 0; m < NV; ++m)
             v[m] = !active ? make_float2(0.f, 0.f) : a.init ? make_float2(a.init_val, 0.f) : buf[t + NT * m];
         __syncwarp();                              // the row is in registers before buf is reused
-        if (a.do_ifft) fft512<true>(v, buf, t, tw2);
+        if (a.do_ifft) hw::fft_row<H, true>(v, buf, t, tw2);
         if (a.v_pre) {
 #pragma unroll
             for (int m = 0; m < NV; ++m) v[m] = c_mul(v[m], tt[t + NT * m]);
@@ -394,7 +414,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_pass_hw512_kernel(MsPlan plan
         if (e1 > e0) {
             // the stash: the row in buf (free between the transforms), then each
             // crossing window's segment x = ox .. ox + win - 1 (wrapped) copied
-            // from there, 16 consecutive pixels per store; entries (site, u, ox)
+            // from there, NT consecutive pixels per store; entries (site, u, ox)
             // are read one per lane and passed round the half-warp
 #pragma unroll
             for (int m = 0; m < NV; ++m) buf[t + NT * m] = v[m];
@@ -421,7 +441,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_pass_hw512_kernel(MsPlan plan
 #pragma unroll
             for (int m = 0; m < NV; ++m) v[m] = c_mul(v[m], tt[t + NT * m]);
         }
-        if (a.do_fft) fft512<false>(v, buf, t, tw2);
+        if (a.do_fft) hw::fft_row<H, false>(v, buf, t, tw2);
         __syncwarp();                              // buf's last reads are done
         entries(y + ystep, e0, e1);
         if (y + ystep < plan.ny) prefetch(y + ystep, slot ^ 1);
@@ -579,20 +599,20 @@ cudaError_t launch_row(const MsPlan& p, const MsRowArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_row_hw512(const MsPlan& p, const MsRowArgs& a, cudaStream_t s) {
-    using namespace hw512;
-    const int groups = (p.ncol + RPB - 1) / RPB;
-    const size_t sm = ((size_t)RPB * ROWBUF + NTW + 2 * N) * sizeof(float2);
+template <int LEN>
+cudaError_t launch_row_hw(const MsPlan& p, const MsRowArgs& a, cudaStream_t s) {
+    using H = hw::Row<LEN>;
+    const int groups = (p.ncol + H::RPB - 1) / H::RPB;
     static std::atomic<bool> attr{false};
     static int per_sm = 0, sms = 0;              // written once, before attr is set
     const cudaError_t e0 = bip_set_once(attr, [&] {
-        cudaError_t e = cudaFuncSetAttribute(row_pass_hw512_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sm);
+        cudaError_t e = cudaFuncSetAttribute(row_pass_hw_kernel<LEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)H::SMEM);
         int dev = 0;
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, row_pass_hw512_kernel, kThreads, sm);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, row_pass_hw_kernel<LEN>, H::THREADS, H::SMEM);
         if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
         return e;
     });
@@ -602,7 +622,7 @@ cudaError_t launch_row_hw512(const MsPlan& p, const MsRowArgs& a, cudaStream_t s
     long long blocks = (long long)sms * per_sm / groups * groups;
     if (blocks < groups) blocks = groups;
     if (blocks > (long long)groups * p.ny) blocks = (long long)groups * p.ny;
-    row_pass_hw512_kernel<<<(unsigned)blocks, kThreads, sm, s>>>(p, a, groups);
+    row_pass_hw_kernel<LEN><<<(unsigned)blocks, H::THREADS, H::SMEM, s>>>(p, a, groups);
     return cudaGetLastError();
 }
 
@@ -627,9 +647,13 @@ cudaError_t bip_ms_row_pass(const MsPlan& p, const MsRowArgs& a, cudaStream_t s)
     switch (p.nx) {
         case 64: return launch_row<64>(p, a, s);
         case 128: return launch_row<128>(p, a, s);
-        case 256: return launch_row<256>(p, a, s);
-        case 512: return p.tw512 ? launch_row_hw512(p, a, s) : launch_row<512>(p, a, s);
-        case 1024: return launch_row<1024>(p, a, s);
+        // 256: the cube's sweeps (2048 columns: 472 -> 355 us per launch).  Parent
+        // sets stay with the radix-8 pass, 1.3% of a fit step slower: other last
+        // bits of their stashes draw the reverse pass's split-BF16 roundings anew
+        // (2.6e-5 of dL/dV).
+        case 256: return p.twhw && p.ncol >= 128 ? launch_row_hw<256>(p, a, s) : launch_row<256>(p, a, s);
+        case 512: return p.twhw ? launch_row_hw<512>(p, a, s) : launch_row<512>(p, a, s);
+        case 1024: return p.twhw ? launch_row_hw<1024>(p, a, s) : launch_row<1024>(p, a, s);
         case 192: return launch_row<192>(p, a, s);
         case 384: return launch_row<384>(p, a, s);
         case 768: return launch_row<768>(p, a, s);
