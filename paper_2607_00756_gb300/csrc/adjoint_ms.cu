@@ -20,6 +20,8 @@
 //   dtbar_p = sum_t w_tp (Ubar_t + dL/dA_t dt_p / (2 |dt_p|))
 // in two deterministic passes: per target (recompute U and A from the
 // stash), then per parent over the targets that use it.
+#include <algorithm>
+
 #include "bip_device.cuh"
 #include "bip_internal.h"
 #include "fft_smem.cuh"
@@ -182,6 +184,11 @@ __global__ void gv_reduce_kernel(const float* part, int groups, int G, float* gV
     gV[i] = s;
 }
 
+__global__ void gv_add_kernel(const float* __restrict__ a, size_t n, float* __restrict__ gV) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        gV[i] += __ldg(&a[i]);
+}
+
 // pass 1: per (target, pixel): Ubar and dL/dA.  Block: 64 window pixels of one
 // site and 64 targets; the parents' values and magnitudes at those pixels are
 // staged in shared memory once (every target reads a few of them), a warp
@@ -326,6 +333,12 @@ cudaError_t bip_ms_adj_row_pass(const MsPlan& p, const MsAdjArgs& a, int* groups
 
 cudaError_t bip_gv_reduce(const float* part, int groups, int G, float* gV, cudaStream_t s) {
     gv_reduce_kernel<<<(G + 255) / 256, 256, 0, s>>>(part, groups, G, gV);
+    return cudaGetLastError();
+}
+
+cudaError_t bip_gv_add(const float* a, size_t n, float* gV, cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    gv_add_kernel<<<(int)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(a, n, gV);
     return cudaGetLastError();
 }
 

@@ -67,8 +67,8 @@ struct bip_ctx {
     bool s1 = false, s2 = false;
 
     DevBuf stash1, stash2, cols;
-    DevBuf cols2;                       // S2's columns while both sweeps run at once (bip_build)
-    cudaStream_t side = nullptr;        // bip_build: the stream S2's sweep runs on
+    DevBuf cols2;                       // S2's columns while both sweeps run at once
+    cudaStream_t side = nullptr;        // the stream S2's sweep runs on (bip_build, the adjoint sweeps)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     DevBuf twhw;                        // the half-warp row pass's twiddles
 
@@ -80,7 +80,8 @@ struct bip_ctx {
     DevBuf occ_d;                       // site occupancies weighting the site sum
     int occ_n = 0;                      // sites they were given for (0: none)
     DevBuf g_s1, g_w, g_R, g_gmt, g_T, g_D, g_Dsum;   // gradient pass workspaces
-    DevBuf g_s1bar, g_s2bar, g_ubar, g_dA, g_dt1, g_dt2, g_adj, g_ckpt, g_seg, g_gvp;
+    DevBuf g_s1bar, g_s2bar, g_ubar, g_dA, g_dt1, g_dt2, g_dV2;
+    DevBuf g_adj[2], g_ckpt[2], g_seg[2], g_gvp[2];   // of the two adjoint sweeps, which run side by side
     DevBuf gpart;                       // parts of a split k range (cgemm_f32.cu)
     DevBuf g_tA, g_tB, g_sA2, g_sB2;    // split-BF16 operands of the reverse-pass contractions
     DevBuf cubeA, cubeB, cube_work, cube_mask;   // the cube on tcgen05
@@ -670,6 +671,14 @@ bip_status build_common(bip_ctx* c, const float* V, const bip_atom* atoms, int32
 }
 
 
+// The stream the second of two sweeps runs on, and its fork and join events.
+bip_status make_side(bip_ctx* c) {
+    if (!c->side) CUDA_TRY(c, cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+    if (!c->ev_fork) CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+    if (!c->ev_join) CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+    return BIP_OK;
+}
+
 // Workspaces of the S1 build: its stash, the column set, the transmissions.
 bip_status alloc_s1(bip_ctx* c, cudaStream_t s) {
     const bip_config& g = c->cfg;
@@ -821,7 +830,8 @@ bip_status bip_destroy(bip_ctx* c) {
                      &c->cube_scratch, &c->bin_of_d, &c->op8A, &c->op8B, &c->f8pmax, &c->f8inv0, &c->f8inv1,
                      &c->f8hmax, &c->f8H, &c->f8sA, &c->f8sB, &c->occ_d, &c->g_s1, &c->g_w, &c->g_R,
                      &c->g_gmt, &c->g_T, &c->g_D, &c->g_Dsum, &c->g_s1bar, &c->g_s2bar, &c->g_ubar, &c->g_dA,
-                     &c->g_dt1, &c->g_dt2, &c->g_adj, &c->g_ckpt, &c->g_seg, &c->g_gvp, &c->pyc, &c->pxc,
+                     &c->g_dt1, &c->g_dt2, &c->g_dV2, &c->g_adj[0], &c->g_ckpt[0], &c->g_seg[0], &c->g_gvp[0],
+                     &c->g_adj[1], &c->g_ckpt[1], &c->g_seg[1], &c->g_gvp[1], &c->pyc, &c->pxc,
                      &c->ray, &c->rax, &c->g_tA, &c->g_tB, &c->g_sA2, &c->g_sB2, &c->cubeA, &c->cubeB,
                      &c->cube_work, &c->cube_mask, &c->s1t, &c->psi, &c->ybuf, &c->cube_grp, &c->cube_wmap, &c->mpart,
                      &c->hcube, &c->shcube, &c->cstash, &c->ccols, &c->xopA, &c->xopB, &c->xm32, &c->tcache,
@@ -922,9 +932,8 @@ bip_status bip_build(bip_ctx* c, const float* V, const bip_atom* atoms, int32_t 
     st = alloc_s1(c, s);
     if (st == BIP_OK) st = alloc_s2(c, c->cols2, s);
     if (st != BIP_OK) return st;
-    if (!c->side) CUDA_TRY(c, cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
-    if (!c->ev_fork) CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-    if (!c->ev_join) CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+    st = make_side(c);
+    if (st != BIP_OK) return st;
     // the transmissions of every slice, once, before the fork (both sweeps read them)
     const size_t G = (size_t)c->cfg.ny * c->cfg.nx;
     TIMED(c, BIP_STAGE_TRANSMISSION, s, bip_transmission(V, (float)c->geo.sigma, 0, c->cfg.nz, G,
@@ -1231,10 +1240,41 @@ int isqrt_up(int n) {
     return k;
 }
 
+// Workspaces `set` of an adjoint sweep over n slices of ncol columns, its
+// checkpoints every ceil(sqrt(n)) slices.
+bip_status adjoint_alloc(bip_ctx* c, int set, int ncol, int n, cudaStream_t s) {
+    const size_t G = (size_t)c->cfg.ny * c->cfg.nx, state = (size_t)ncol * G;
+    const int k = isqrt_up(n), nck = (n + k - 1) / k;
+    CUDA_TRY(c, ensure(set ? c->cols2 : c->cols, state * sizeof(float2), false, s));
+    CUDA_TRY(c, ensure(c->g_adj[set], state * sizeof(float2), false, s));
+    CUDA_TRY(c, ensure(c->g_ckpt[set], (size_t)nck * state * sizeof(float2), false, s));
+    CUDA_TRY(c, ensure(c->g_seg[set], (size_t)k * state * sizeof(float2), false, s));
+    CUDA_TRY(c, ensure(c->g_gvp[set], (size_t)ncol * G * sizeof(float), false, s));
+    return BIP_OK;
+}
+
+// Whether S2's adjoint sweep can have workspaces of its own beside S1's: they
+// are there already, or the device has twice their size free.
+bool adjoint_pair_fits(bip_ctx* c, int ncol, int n) {
+    const size_t G = (size_t)c->cfg.ny * c->cfg.nx, state = (size_t)ncol * G * sizeof(float2);
+    const int k = isqrt_up(n), nck = (n + k - 1) / k;
+    const size_t nv = (size_t)c->cfg.nz * G;
+    if (c->cols2.cap >= state && c->g_adj[1].cap >= state && c->g_ckpt[1].cap >= nck * state &&
+        c->g_seg[1].cap >= k * state && c->g_gvp[1].cap >= state / 2 && c->tcache.cap >= nv * sizeof(float2) &&
+        c->g_dV2.cap >= nv * sizeof(float))
+        return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return free_b / 2 >= (size_t)(nck + k + 3) * state + 3 * nv * sizeof(float);
+}
+
 // dL/dV_j through the S1 sweep (psi_{j+1} = Prop(T_j psi_j)), j < the last
 // ionization plane, from the window adjoints dtbar1 of every site; forward
 // states recomputed from checkpoints every ceil(sqrt(n)) slices
-bip_status adjoint_s1(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
+bip_status adjoint_s1(bip_ctx* c, const float* V, const float2* T, float* dV, cudaStream_t s) {
     const bip_config& g = c->cfg;
     const size_t G = (size_t)g.ny * g.nx;
     const int ncol = c->geo.Bp1;
@@ -1243,15 +1283,11 @@ bip_status adjoint_s1(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
     if (jmax == 0) return BIP_OK;
     const int n = jmax, k = isqrt_up(n), nck = (n + k - 1) / k;
     const size_t state = (size_t)ncol * G;
-    CUDA_TRY(c, ensure(c->g_adj, state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_ckpt, (size_t)nck * state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_seg, (size_t)k * state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_gvp, (size_t)ncol * G * sizeof(float), false, s));
     MsPlan fp = plan_for(c, ncol, c->shift1), cp = fp;
     cp.py = (const float2*)c->pyc.p;
     cp.px = (const float2*)c->pxc.p;
     float2* cols = (float2*)c->cols.p;
-    float2* adj = (float2*)c->g_adj.p;
+    float2* adj = (float2*)c->g_adj[0].p;
     auto row_off = [&](int j) -> const int32_t* {
         return c->plane_off[j + 1] > c->plane_off[j] ? (const int32_t*)c->row_off_d.p + (size_t)j * (g.ny + 1) : nullptr;
     };
@@ -1262,6 +1298,7 @@ bip_status adjoint_s1(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
         a.init_val = 1.0f;
         a.do_ifft = j > 0;
         a.v_post = V + (size_t)j * G;
+        a.t_slice = T ? T + (size_t)j * G : nullptr;
         a.do_fft = fft;
         a.win = g.win;
         a.save = save;
@@ -1271,13 +1308,13 @@ bip_status adjoint_s1(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
     const int last_ck = (nck - 1) * k;
     for (int j = 0; j < last_ck; ++j) {
         if (j % k == 0 && j > 0)
-            CUDA_TRY(c, cudaMemcpyAsync((float2*)c->g_ckpt.p + (size_t)(j / k) * state, cols, state * sizeof(float2),
+            CUDA_TRY(c, cudaMemcpyAsync((float2*)c->g_ckpt[0].p + (size_t)(j / k) * state, cols, state * sizeof(float2),
                                         cudaMemcpyDeviceToDevice, s));
         CUDA_TRY(c, fwd_row(j, nullptr, true));
         CUDA_TRY(c, bip_ms_col_pass(fp, cols, s));
     }
     if (last_ck > 0)
-        CUDA_TRY(c, cudaMemcpyAsync((float2*)c->g_ckpt.p + (size_t)(last_ck / k) * state, cols, state * sizeof(float2),
+        CUDA_TRY(c, cudaMemcpyAsync((float2*)c->g_ckpt[0].p + (size_t)(last_ck / k) * state, cols, state * sizeof(float2),
                                     cudaMemcpyDeviceToDevice, s));
     int groups = 0;
     auto adj_row = [&](int j, bool zero_in, const float2* st, bool fft) -> bip_status {
@@ -1293,10 +1330,10 @@ bip_status adjoint_s1(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
         a.row_ent = (const int4*)c->row_ent_d.p;
         a.win = g.win;
         a.inj = (const float2*)c->g_dt1.p;
-        a.gv_part = (float*)c->g_gvp.p;
+        a.gv_part = (float*)c->g_gvp[0].p;
         a.do_fft = fft;
         CUDA_TRY(c, bip_ms_adj_row_pass(fp, a, &groups, s));
-        if (st) CUDA_TRY(c, bip_gv_reduce((const float*)c->g_gvp.p, groups, (int)G, dV + (size_t)j * G, s));
+        if (st) CUDA_TRY(c, bip_gv_reduce((const float*)c->g_gvp[0].p, groups, (int)G, dV + (size_t)j * G, s));
         return BIP_OK;
     };
     // lambda at the last plane: its window adjoints only
@@ -1306,14 +1343,14 @@ bip_status adjoint_s1(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
     for (int m = nck - 1; m >= 0; --m) {
         const int j0 = m * k, j1 = std::min(j0 + k, n) - 1;
         if (m > 0)
-            CUDA_TRY(c, cudaMemcpyAsync(cols, (float2*)c->g_ckpt.p + (size_t)m * state, state * sizeof(float2),
+            CUDA_TRY(c, cudaMemcpyAsync(cols, (float2*)c->g_ckpt[0].p + (size_t)m * state, state * sizeof(float2),
                                         cudaMemcpyDeviceToDevice, s));
         for (int j = j0; j <= j1; ++j) {
-            CUDA_TRY(c, fwd_row(j, (float2*)c->g_seg.p + (size_t)(j - j0) * state, j < j1));
+            CUDA_TRY(c, fwd_row(j, (float2*)c->g_seg[0].p + (size_t)(j - j0) * state, j < j1));
             if (j < j1) CUDA_TRY(c, bip_ms_col_pass(fp, cols, s));
         }
         for (int j = j1; j >= j0; --j) {
-            st = adj_row(j, false, (const float2*)c->g_seg.p + (size_t)(j - j0) * state, j > 0);
+            st = adj_row(j, false, (const float2*)c->g_seg[0].p + (size_t)(j - j0) * state, j > 0);
             if (st != BIP_OK) return st;
             if (j > 0) CUDA_TRY(c, bip_ms_col_pass(cp, adj, s));
         }
@@ -1323,7 +1360,7 @@ bip_status adjoint_s1(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
 
 // dL/dV_j through the S2 sweep (x_j = T_j Prop(x_{j+1})), j >= the first
 // ionization plane, ascending, from the window adjoints dtbar2
-bip_status adjoint_s2(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
+bip_status adjoint_s2(bip_ctx* c, const float* V, const float2* T, int set, float* dV, cudaStream_t s) {
     const bip_config& g = c->cfg;
     const size_t G = (size_t)g.ny * g.nx;
     const int ncol = c->geo.Bp2;
@@ -1332,15 +1369,11 @@ bip_status adjoint_s2(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
     if (first >= g.nz) return BIP_OK;
     const int n = g.nz - first, k = isqrt_up(n), nck = (n + k - 1) / k;
     const size_t state = (size_t)ncol * G;
-    CUDA_TRY(c, ensure(c->g_adj, state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_ckpt, (size_t)nck * state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_seg, (size_t)k * state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_gvp, (size_t)ncol * G * sizeof(float), false, s));
     MsPlan fp = plan_for(c, ncol, c->shift2), cp = fp;
     cp.py = (const float2*)c->pyc.p;
     cp.px = (const float2*)c->pxc.p;
-    float2* cols = (float2*)c->cols.p;
-    float2* adj = (float2*)c->g_adj.p;
+    float2* cols = (float2*)(set ? c->cols2 : c->cols).p;
+    float2* adj = (float2*)c->g_adj[set].p;
     auto row_off = [&](int j) -> const int32_t* {
         return c->plane_off[j + 1] > c->plane_off[j] ? (const int32_t*)c->row_off_d.p + (size_t)j * (g.ny + 1) : nullptr;
     };
@@ -1349,6 +1382,7 @@ bip_status adjoint_s2(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
         a.cols = cols;
         a.do_ifft = 1;
         a.v_pre = V + (size_t)j * G;
+        a.t_slice = T ? T + (size_t)j * G : nullptr;
         a.do_fft = fft;
         a.win = g.win;
         a.save = save;
@@ -1369,7 +1403,7 @@ bip_status adjoint_s2(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
     const int lowest_ck = g.nz - 1 - (nck - 1) * k;
     for (int j = g.nz - 1; j >= lowest_ck; --j) {
         if ((g.nz - 1 - j) % k == 0)
-            CUDA_TRY(c, cudaMemcpyAsync((float2*)c->g_ckpt.p + (size_t)((g.nz - 1 - j) / k) * state, cols,
+            CUDA_TRY(c, cudaMemcpyAsync((float2*)c->g_ckpt[set].p + (size_t)((g.nz - 1 - j) / k) * state, cols,
                                         state * sizeof(float2), cudaMemcpyDeviceToDevice, s));
         if (j == lowest_ck) break;
         CUDA_TRY(c, fwd_row(j, nullptr, true));
@@ -1378,10 +1412,10 @@ bip_status adjoint_s2(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
     int groups = 0;
     for (int m = nck - 1; m >= 0; --m) {
         const int jhi = g.nz - 1 - m * k, jlo = std::max(first, jhi - k + 1);
-        CUDA_TRY(c, cudaMemcpyAsync(cols, (float2*)c->g_ckpt.p + (size_t)m * state, state * sizeof(float2),
+        CUDA_TRY(c, cudaMemcpyAsync(cols, (float2*)c->g_ckpt[set].p + (size_t)m * state, state * sizeof(float2),
                                     cudaMemcpyDeviceToDevice, s));
         for (int j = jhi; j >= jlo; --j) {
-            CUDA_TRY(c, fwd_row(j, (float2*)c->g_seg.p + (size_t)(j - jlo) * state, j > jlo));
+            CUDA_TRY(c, fwd_row(j, (float2*)c->g_seg[set].p + (size_t)(j - jlo) * state, j > jlo));
             if (j > jlo) CUDA_TRY(c, bip_ms_col_pass(fp, cols, s));
         }
         for (int j = jlo; j <= jhi; ++j) {
@@ -1390,17 +1424,17 @@ bip_status adjoint_s2(bip_ctx* c, const float* V, float* dV, cudaStream_t s) {
             a.zero_in = j == first;
             a.do_ifft = j > first;
             a.v = V + (size_t)j * G;
-            a.state = (const float2*)c->g_seg.p + (size_t)(j - jlo) * state;
+            a.state = (const float2*)c->g_seg[set].p + (size_t)(j - jlo) * state;
             a.state_times_T = 0;
             a.inj_before = 1;
             a.row_off = row_off(j);
             a.row_ent = (const int4*)c->row_ent_d.p;
             a.win = g.win;
             a.inj = (const float2*)c->g_dt2.p;
-            a.gv_part = (float*)c->g_gvp.p;
+            a.gv_part = (float*)c->g_gvp[set].p;
             a.do_fft = j < g.nz - 1;
             CUDA_TRY(c, bip_ms_adj_row_pass(fp, a, &groups, s));
-            CUDA_TRY(c, bip_gv_reduce((const float*)c->g_gvp.p, groups, (int)G, dV + (size_t)j * G, s));
+            CUDA_TRY(c, bip_gv_reduce((const float*)c->g_gvp[set].p, groups, (int)G, dV + (size_t)j * G, s));
             if (j < g.nz - 1) CUDA_TRY(c, bip_ms_col_pass(cp, adj, s));
         }
     }
@@ -3045,8 +3079,8 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
     const size_t perA = (size_t)Dpad * K, perB = (size_t)nch * Bpad * K, perS1 = (size_t)Bpad * K;
     const size_t ldm = (size_t)nch * Dpad, perMt = (size_t)Bpad * ldm, perQ = (size_t)Bpad * Bpad;
     const size_t perT = (size_t)nch * Bpad * K;
-    // contractions of the reverse pass on the tensor cores (split BF16, three
-    // products) for the tensor-core precisions, FP32 SIMT for FP32
+    // the large contractions of the reverse pass in split BF16 (three products)
+    // for the tensor-core precisions, in FP32 (three BF16 terms) for FP32
     const bool tcg = c->prec != BIP_PREC_FP32;
     const int D128 = round_up(Dpad, 128);
     const size_t KB = (size_t)nch * Bpad;
@@ -3318,11 +3352,47 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
         if (st != BIP_OK) return st;
     }
     if (d_V) {
-        CUDA_TRY(c, cudaMemsetAsync(d_V, 0, (size_t)g.nz * g.ny * g.nx * sizeof(float), s));
-        st = adjoint_s1(c, V, d_V, s);
+        // The two sweeps side by side (as bip_build's: their launches of a few
+        // columns leave most of the chip idle), S2's derivative in a buffer of
+        // its own that is added at the end: the sums and their order are those
+        // of one sweep after the other, which a device with little memory left
+        // still runs.  Everything written is allocated before they fork.  256^2,
+        // 40 slices, 64 sites, build to derivatives: 30.0 -> 28.8 ms (mixed), 54.1 ->
+        // 53.1 (FP32).
+        const size_t G = (size_t)g.ny * g.nx, nv = (size_t)g.nz * G;
+        int jmax = 0, first = g.nz;
+        for (auto& sd : c->sites) {
+            jmax = std::max(jmax, (int)sd.plane);
+            first = std::min(first, (int)sd.plane);
+        }
+        const int n2 = g.nz - first;
+        const bool pair = jmax > 0 && n2 > 0 && adjoint_pair_fits(c, geo.Bp2, n2);
+        st = jmax > 0 ? adjoint_alloc(c, 0, geo.Bp1, jmax, s) : BIP_OK;
+        if (st == BIP_OK && n2 > 0) st = adjoint_alloc(c, pair ? 1 : 0, geo.Bp2, n2, s);
         if (st != BIP_OK) return st;
-        st = adjoint_s2(c, V, d_V, s);
-        if (st != BIP_OK) return st;
+        CUDA_TRY(c, cudaMemsetAsync(d_V, 0, nv * sizeof(float), s));
+        if (pair) {
+            CUDA_TRY(c, ensure(c->tcache, nv * sizeof(float2), false, s));
+            CUDA_TRY(c, ensure(c->g_dV2, nv * sizeof(float), false, s));
+            st = make_side(c);
+            if (st != BIP_OK) return st;
+            const float2* T = (const float2*)c->tcache.p;
+            CUDA_TRY(c, bip_transmission(V, (float)geo.sigma, 0, g.nz, G, (float2*)c->tcache.p, s));
+            CUDA_TRY(c, cudaMemsetAsync(c->g_dV2.p, 0, nv * sizeof(float), s));
+            CUDA_TRY(c, cudaEventRecord(c->ev_fork, s));
+            CUDA_TRY(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+            // the caller's stream waits for S2 whatever happened
+            const bip_status st2 = adjoint_s2(c, V, T, 1, (float*)c->g_dV2.p, c->side);
+            const bip_status st1 = st2 == BIP_OK ? adjoint_s1(c, V, T, d_V, s) : st2;
+            CUDA_TRY(c, cudaEventRecord(c->ev_join, c->side));
+            CUDA_TRY(c, cudaStreamWaitEvent(s, c->ev_join, 0));
+            if (st1 != BIP_OK) return st1;
+            CUDA_TRY(c, bip_gv_add((const float*)c->g_dV2.p, nv, d_V, s));
+        } else {
+            st = adjoint_s1(c, V, nullptr, d_V, s);
+            if (st == BIP_OK) st = adjoint_s2(c, V, nullptr, 0, d_V, s);
+            if (st != BIP_OK) return st;
+        }
     }
     if (d_aberr) {
         std::vector<double2> D(B);
