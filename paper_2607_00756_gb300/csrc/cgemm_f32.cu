@@ -37,7 +37,8 @@
 // tile where its MMAs take 12 x 128.  Measured on 19 x 1024 x 1024 x 4096:
 // 220 TFLOP/s of complex products (SIMT FFMA, 64 x 64 tiles: 47); two groups
 // of four cutting warps taking chunks in turn 209-218, sixteen cutting warps
-// of 40 registers 160, loads issued between the cutting of A and of B 219.
+// of 40 registers 160, loads issued between the cutting of A and of B 219, two
+// CTAs sharing a tile of 256 rows (cta_group::2, each with half of B) 192-212.
 //
 // Units: (batch, tile of 128 rows, tile of nt columns, k range).  Where the
 // tiles alone leave SMs idle the k range is split (cgemm_plan), each part
@@ -151,20 +152,20 @@ struct Slot {
     __device__ int k_of(int i) const { return KC ? k + (i & 1) : k + 8 * (i >> 2) + (i & 3); }
 };
 
-// the thread's eight values of chunk `step`, rows row0 + its slot's (zeros
-// past the last k).  Rows past the last are clamped to it: what they give
-// reaches only rows of C that are not written.
+// the thread's eight values of chunk `step` of the tile whose first row is at
+// base (zeros past the last k).  Rows past the last of `rows` are clamped to
+// it: what they give reaches only rows of C that are not written.
 template <bool KC>
-__device__ __forceinline__ void load8(float2 (&v)[8], const CGemmOperand& o, const float2* base, int row0, int rows,
+__device__ __forceinline__ void load8(float2 (&v)[8], const CGemmOperand& o, const float2* base, int rows,
                                       const Slot<KC>& sl, int step) {
     // block kb of the two-level k axis
     const int k0 = step * kStep;
     const int kb = o.nper > 1 ? k0 / o.kper : 0;
     const int kin = k0 - kb * o.kper;
-    const float2* src = base + (int64_t)kb * o.sk2 + (KC ? kin + sl.k : (kin + sl.k) * (int)o.sk);
+    const float2* src = base + (int64_t)kb * o.sk2 + (KC ? kin + sl.k : (kin + sl.k) * o.sk);
     int off[4];
 #pragma unroll
-    for (int i = 0; i < (KC ? 4 : 1); ++i) off[i] = min(row0 + sl.row_of(2 * i), rows - 1) * (KC ? (int)o.sr : 1);
+    for (int i = 0; i < (KC ? 4 : 1); ++i) off[i] = min(sl.row_of(2 * i), rows - 1) * (KC ? (int)o.sr : 1);
     if (kin + kStep <= o.kvalid) {
         if (KC && o.vec) {
 #pragma unroll
@@ -412,8 +413,8 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
         int st = u.s0;
         float2 va[8], vb[8];
         auto load = [&]() {
-            load8<AKC>(va, p.A, p.A.p + (int64_t)u.z * p.A.sb, u.m0, p.M, sla, st);
-            load8<BKC>(vb, p.B, p.B.p + (int64_t)u.z * p.B.sb, u.n0, u.n1, slb, st);
+            load8<AKC>(va, p.A, p.A.p + u.z * p.A.sb + u.m0 * p.A.sr, p.M - u.m0, sla, st);
+            load8<BKC>(vb, p.B, p.B.p + u.z * p.B.sb + u.n0 * p.B.sr, u.n1 - u.n0, slb, st);
             if (p.dk) {
                 const float* w = p.dk + (int64_t)u.z * p.sdb;
 #pragma unroll
@@ -589,9 +590,8 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
         o->kper = (o->kvalid + kStep - 1) / kStep * kStep;
         o->vec = o->sk == 1 && aligned2(o->p, o->sr, o->sk2, o->sb);
         if (o->sk != 1 && o->sr != 1) return cudaErrorInvalidValue;
-        // offsets within a sheet are 32-bit in the kernel
-        const int64_t rows = o == &p.A ? p.M : p.N;
-        if ((rows - 1) * o->sr + (int64_t)(o->kper + kStep) * o->sk > 0x7fffffff) return cudaErrorInvalidValue;
+        // offsets within a tile's chunk are 32-bit in the kernel
+        if (127 * o->sr + kStep > 0x7fffffff || kStep * o->sk > 0x7fffffff) return cudaErrorInvalidValue;
     }
     if (p.A.kvalid != p.B.kvalid || p.A.nper != p.B.nper) return cudaErrorInvalidValue;
     if (p.dk && p.A.nper != 1) return cudaErrorInvalidValue;

@@ -121,3 +121,26 @@ def test_repeats_bit_for_bit_and_keeps_nonfinite_rows_apart(env):
     rows[[5, 129]] = False
     assert torch.all(fine[rows]) and not torch.any(fine[~rows])
     assert torch.equal(torch.view_as_real(bad[0][rows]), torch.view_as_real(C[0][0][rows]))
+
+
+@pytest.mark.parametrize("layout", ["k", "r"])
+def test_operands_of_more_than_31_bits(env, layout):
+    """Rows (or k) 2^24 elements apart: the last lies past 2^31 elements."""
+    capi, ctx = env
+    rng = torch.Generator("cuda").manual_seed(8)
+    far, n, near = 1 << 24, 131, 17
+    M, K = (n, near) if layout == "k" else (near, n)
+    a = torch.randn(M, K, dtype=torch.complex64, device="cuda", generator=rng)
+    t = torch.empty((n - 1) * far + near, dtype=torch.complex64, device="cuda")
+    torch.as_strided(t, (n, near), (far, 1)).copy_(a if layout == "k" else a.T)
+    s = (far, 1, 0, 0) if layout == "k" else (1, far, 0, 0)
+    B, sB, b = operand(rng, 40, K, 1, 1, "k", 0)
+    for flags in (0, 8):
+        C = torch.full((M, 40) if flags == 0 else (40, M), float("nan"), dtype=torch.complex64, device="cuda")
+        capi.bip_debug_cgemm(ctx, M, 40, K, 1, 1, t, s, B, sB, flags, None, C)
+        got = C if flags == 0 else C.T
+        a2, b2 = a.to(torch.complex128), b[0]
+        assert torch.all((got - a2 @ b2.T).abs() <= bound(K) * (a2.abs() @ b2.abs().T))
+    C = torch.full((40, M), float("nan"), dtype=torch.complex64, device="cuda")
+    capi.bip_debug_cgemm(ctx, 40, M, K, 1, 1, B, sB, t, s, 0, None, C)
+    assert torch.all((C - b2 @ a2.T).abs() <= bound(K) * (b2.abs() @ a2.abs().T))
