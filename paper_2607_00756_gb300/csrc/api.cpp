@@ -979,8 +979,10 @@ void release_map_workspaces(bip_ctx* c, cudaStream_t s) {
 
 // Waits for the stream and turns the kernels' give-up flag into a status.
 // The flag comes back through pinned memory: a pageable copy waits for the
-// stream and then once more for itself (9 us).
+// stream and then once more for itself (9 us).  An FP32 context's calls can be
+// captured as they are; there the flag is left to bip_check_errors.
 bip_status check_flag(bip_ctx* c, cudaStream_t s) {
+    if (c->prec == BIP_PREC_FP32 && capturing(s)) return BIP_OK;
     CUDA_TRY(c, cudaMemcpyAsync(c->flag_h, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(c, cudaStreamSynchronize(s));
     if (*c->flag_h) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");

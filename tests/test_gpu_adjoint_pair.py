@@ -54,3 +54,42 @@ def test_sweeps_side_by_side(slices):
                 assert np.array_equal(out, first)
         finally:
             ctx.close()
+
+
+@pytest.mark.parametrize("safe", [0, 1])
+def test_fp32_calls_can_be_captured(safe):
+    """An FP32 context's coupling and derivatives (both adjoint sweeps) as a
+    CUDA graph after one call as warm-up, capture-safe or not: a replay gives
+    the call's bits, and the flag of a wait that ran out stays readable."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2607_00756_gb300 import capi
+    from paper_2607_00756_gb300.context import BipContext
+    cfg = synth.config1()
+    sp = synth.make_specimen(cfg)
+    dev = torch.device("cuda:0")
+    V = torch.tensor(sp.V, dtype=torch.float32, device=dev)
+    H = torch.tensor(sp.H, dtype=torch.complex64, device=dev)
+    g = torch.linspace(-1.0, 1.0, len(sp.scans), dtype=torch.float64, device=dev)
+    ctx = BipContext(cfg, prec="fp32")
+    try:
+        ctx.build(V, sp.atoms, sp.nch)
+        capi.bip_set_capture_safe(ctx.ctx, safe)
+
+        def call():
+            d = ctx.grad(H, sp.scans, g, occ=False, aberr=False, V=V)
+            return d["V"], d["H"], ctx.coupling(H, 0)
+
+        want = call()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+            got = call()
+        graph.replay()
+        torch.cuda.synchronize()
+        for a, b in zip(got, want):
+            a, b = (torch.view_as_real(t) if t.is_complex() else t for t in (a, b))
+            assert float(b.abs().max()) > 0 and torch.equal(a, b)
+        capi.bip_check_errors(ctx.ctx)
+    finally:
+        ctx.close()
