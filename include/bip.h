@@ -532,6 +532,15 @@ bip_status bip_debug_cgemm(bip_ctx* ctx, int32_t M, int32_t N, int32_t K, int32_
                            const void* A, const int64_t* sA, const void* B, const int64_t* sB, int32_t flags,
                            const float* w, void* C, void* stream);
 
+/* The split into BF16 planes that feeds the tensor-core contractions of the
+ * cube and the reverse pass, by itself, for validation: dst[plane][i][dcol0 +
+ * k], planes re_hi, re_lo, im_hi, im_lo of rows x d_cols values, from
+ * src[i s_row + k s_col] (complex64 device, one stride 1; conjugated when
+ * conj), i < rows, k < cols; the rest of dst is left as it is.
+ * BIP_ERR_INVALID_ARG for a null pointer, a size below 1 or such strides. */
+bip_status bip_debug_split(bip_ctx* ctx, int32_t rows, int32_t cols, const void* src, int64_t s_row, int64_t s_col,
+                           int32_t d_cols, int32_t dcol0, int32_t conj, void* dst, void* stream);
+
 /* Text of the last error on this context ("" if none; static text if ctx
  * is NULL). */
 const char* bip_last_error(const bip_ctx* ctx);

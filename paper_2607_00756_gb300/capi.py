@@ -70,6 +70,7 @@ def _load():
         "bip_debug_fail_alloc": [ctypes.c_int64],
         "bip_debug_allocs": [P(ctypes.c_int64), P(ctypes.c_int64)],
         "bip_debug_cgemm": [VP, I32, I32, I32, I32, I32, VP, P(ctypes.c_int64), VP, P(ctypes.c_int64), I32, VP, VP, VP],
+        "bip_debug_split": [VP, I32, I32, VP, ctypes.c_int64, ctypes.c_int64, I32, I32, I32, VP, VP],
         "bip_qeels_bins": [VP, I32, P(I32), P(I32)],
         "bip_coreloss_qeels": [VP, VP, P(D), I32, I32, VP, VP],
         "bip_copy_stash": [VP, I32, I32, VP, VP],
@@ -309,6 +310,15 @@ def bip_debug_cgemm(ctx, M, N, K, blocks, batch, A, sA, B, sB, flags, w, C, stre
            _lib.bip_debug_cgemm(ctx, M, N, K, blocks, batch, ctypes.c_void_p(A.data_ptr()), arr(*sA),
                                 ctypes.c_void_p(B.data_ptr()), arr(*sB), flags, _dev(w), _dev(C), _stream(stream)))
     return C
+
+
+def bip_debug_split(ctx, rows, cols, src, s_row, s_col, d_cols, dcol0, conj, dst, stream=None):
+    """The split-BF16 planes of a complex64 CUDA tensor (its storage, addressed
+    by the strides) into dst, bfloat16 [4, rows, d_cols]."""
+    _check("bip_debug_split", ctx,
+           _lib.bip_debug_split(ctx, rows, cols, ctypes.c_void_p(src.data_ptr()), s_row, s_col, d_cols, dcol0,
+                                int(conj), ctypes.c_void_p(dst.data_ptr()), _stream(stream)))
+    return dst
 
 
 def bip_debug_allocs():
