@@ -267,7 +267,7 @@ bip_status bip_coreloss_sites(bip_ctx* ctx, const void* H, const double* scan_px
  *   H, scan_px as bip_coreloss_map.
  *   cube_out [P, n_cube] float32 device, overwritten; beams in the order of
  *            bip_cube_beams.
- * Precisions: the coupling M in the context's precision -- FP32 (SIMT),
+ * Precisions: the coupling M in the context's precision -- FP32,
  * SPLIT_BF16 and MIXED (tcgen05); FP8 contexts return BIP_ERR_UNSUPPORTED.
  * The per-beam sum over b: on a raster scan list (scan p = my Mx + mx at
  * (ry[my], rx[mx])) separated over the aperture beams' lattice, two short
