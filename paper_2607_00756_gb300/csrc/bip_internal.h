@@ -319,7 +319,7 @@ struct CGemmF32 {
     int* err;
     uint64_t wait_ns;
     // (plan)
-    int nt, n_tiles, ch_tiles, tiles, steps, ksplit, units, vecC;
+    int cols, nt, n_tiles, tiles, steps, ksplit, units, vecC;   // cols: columns of C computed
 };
 // fills the plan; *part_elems: float2 elements `part` must hold (0: none)
 cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems);

@@ -116,14 +116,8 @@ __device__ __forceinline__ bool unit_of(const CGemmF32& p, int i, Unit& u) {
         u.m0 = r / p.n_tiles * 128;
         r %= p.n_tiles;
     }
-    if (p.ep_B > 0) {
-        // the tiles of a channel's ep_n columns
-        u.n0 = r / p.ch_tiles * p.ep_B + r % p.ch_tiles * p.nt;
-        u.n1 = min(u.n0 + p.nt, r / p.ch_tiles * p.ep_B + p.ep_n);
-    } else {
-        u.n0 = r * p.nt;
-        u.n1 = min(u.n0 + p.nt, p.N);
-    }
+    u.n0 = r * p.nt;
+    u.n1 = min(u.n0 + p.nt, p.cols);
     u.s0 = (int)((int64_t)p.steps * u.ks / p.ksplit);
     u.s1 = (int)((int64_t)p.steps * (u.ks + 1) / p.ksplit);
     return true;
@@ -152,33 +146,38 @@ struct Slot {
     __device__ int k_of(int i) const { return KC ? k + (i & 1) : k + 8 * (i >> 2) + (i & 3); }
 };
 
-// the thread's eight values of chunk `step` of the tile whose first row is at
-// base (zeros past the last k).  Rows past the last of `rows` are clamped to
-// it: what they give reaches only rows of C that are not written.
+// row of B that column n of C comes from
+__device__ __forceinline__ int row_of_column(const CGemmF32& p, int n) {
+    return p.ep_B > 0 ? n / p.ep_n * p.ep_B + n % p.ep_n : n;
+}
+
+// the thread's eight values of chunk `step`, of its rows row[] (zeros past the
+// last k).  Rows past the last were clamped to it: what they give reaches only
+// rows and columns of C that are not written.
 template <bool KC>
-__device__ __forceinline__ void load8(float2 (&v)[8], const CGemmOperand& o, const float2* base, int rows,
-                                      const Slot<KC>& sl, int step) {
+__device__ __forceinline__ void load8(float2 (&v)[8], const CGemmOperand& o, const float2* base,
+                                      const int (&row)[KC ? 4 : 1], const Slot<KC>& sl, int step) {
     // block kb of the two-level k axis
     const int k0 = step * kStep;
     const int kb = o.nper > 1 ? k0 / o.kper : 0;
     const int kin = k0 - kb * o.kper;
-    const float2* src = base + (int64_t)kb * o.sk2 + (KC ? kin + sl.k : (kin + sl.k) * o.sk);
-    int off[4];
+    const float2* src = base + (int64_t)kb * o.sk2 + (KC ? kin + sl.k : (int64_t)(kin + sl.k) * (int)o.sk);
+    const float2* at[KC ? 4 : 1];
 #pragma unroll
-    for (int i = 0; i < (KC ? 4 : 1); ++i) off[i] = min(sl.row_of(2 * i), rows - 1) * (KC ? (int)o.sr : 1);
+    for (int i = 0; i < (KC ? 4 : 1); ++i) at[i] = src + (KC ? (int64_t)row[i] * (int)o.sr : row[i]);
     if (kin + kStep <= o.kvalid) {
         if (KC && o.vec) {
 #pragma unroll
             for (int i = 0; i < 8; i += 2) {
-                const float4 f = __ldg(reinterpret_cast<const float4*>(src + off[i / 2]));
+                const float4 f = __ldg(reinterpret_cast<const float4*>(at[KC ? i / 2 : 0]));
                 v[i] = make_float2(f.x, f.y);
                 v[i + 1] = make_float2(f.z, f.w);
             }
         } else if (KC) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = __ldg(src + off[i / 2] + (i & 1));
+            for (int i = 0; i < 8; ++i) v[i] = __ldg(at[KC ? i / 2 : 0] + (i & 1));
         } else {
-            const float2* q = src + off[0];
+            const float2* q = at[0];
 #pragma unroll
             for (int i = 0; i < 8; ++i) v[i] = __ldg(q + ((i >> 2) * 8 + (i & 3)) * (int)o.sk);
         }
@@ -187,7 +186,7 @@ __device__ __forceinline__ void load8(float2 (&v)[8], const CGemmOperand& o, con
         for (int i = 0; i < 8; ++i) {
             v[i] = make_float2(0.f, 0.f);
             if (kin + sl.k_of(i) < o.kvalid)
-                v[i] = __ldg(KC ? src + off[i / 2] + (i & 1) : src + off[0] + ((i >> 2) * 8 + (i & 3)) * (int)o.sk);
+                v[i] = __ldg(KC ? at[KC ? i / 2 : 0] + (i & 1) : at[0] + ((i >> 2) * 8 + (i & 3)) * (int)o.sk);
         }
     }
 }
@@ -293,7 +292,7 @@ __device__ __forceinline__ float2 unpack2(uint64_t v) {
 __device__ __forceinline__ int64_t out_at(const CGemmF32& p, int z, int m, int n) {
     int64_t o = (int64_t)z * p.scb;
     if (p.ep_B > 0)                              // the coupling as the Gram operand: n = (ch, b), m = d
-        return o + (int64_t)(n % p.ep_B) * p.scn + (int64_t)(n / p.ep_B) * p.ep_Dp + m;
+        return o + (int64_t)(n % p.ep_n) * p.scn + (int64_t)(n / p.ep_n) * p.ep_Dp + m;
     return o + (int64_t)m * p.scm + (int64_t)n * p.scn;
 }
 
@@ -412,9 +411,18 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
         bool more = unit_of(p, 0, u);
         int st = u.s0;
         float2 va[8], vb[8];
+        int rb[BKC ? 4 : 1];
+        auto rows = [&]() {
+#pragma unroll
+            for (int j = 0; j < (BKC ? 4 : 1); ++j)
+                rb[j] = row_of_column(p, min(u.n0 + slb.row_of(2 * j), u.n1 - 1));
+        };
         auto load = [&]() {
-            load8<AKC>(va, p.A, p.A.p + u.z * p.A.sb + u.m0 * p.A.sr, p.M - u.m0, sla, st);
-            load8<BKC>(vb, p.B, p.B.p + u.z * p.B.sb + u.n0 * p.B.sr, u.n1 - u.n0, slb, st);
+            int ra[AKC ? 4 : 1];
+#pragma unroll
+            for (int j = 0; j < (AKC ? 4 : 1); ++j) ra[j] = min(u.m0 + sla.row_of(2 * j), p.M - 1);
+            load8<AKC>(va, p.A, p.A.p + u.z * p.A.sb, ra, sla, st);
+            load8<BKC>(vb, p.B, p.B.p + u.z * p.B.sb, rb, slb, st);
             if (p.dk) {
                 const float* w = p.dk + (int64_t)u.z * p.sdb;
 #pragma unroll
@@ -426,7 +434,10 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
                 }
             }
         };
-        if (more) load();
+        if (more) {
+            rows();
+            load();
+        }
         int s = 0;
         uint32_t ph = 0;
 #pragma unroll 1
@@ -451,6 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
             if (++st == u.s1) {
                 more = unit_of(p, ++i, u);
                 st = u.s0;
+                if (more) rows();
             }
             if (more) load();
         }
@@ -498,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
             float2* o;
             bool vec = false;
             if (p.ksplit > 1) {
-                o = p.part + (((int64_t)u.ks * p.batch + u.z) * p.M + m) * p.N + n0;
+                o = p.part + (((int64_t)u.ks * p.batch + u.z) * p.M + m) * p.cols + n0;
             } else {
                 o = p.C + out_at(p, u.z, m, n0);
                 vec = p.vecC;
@@ -532,14 +544,13 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
 
 // C from the parts of a split k range, added in order
 __global__ void __launch_bounds__(256) cgemm_sum_kernel(const CGemmF32 p) {
-    const int64_t n_el = (int64_t)p.batch * p.M * p.N;
+    const int64_t n_el = (int64_t)p.batch * p.M * p.cols;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n_el) return;
-    const int n = (int)(i % p.N);
-    const int64_t zm = i / p.N;
+    const int n = (int)(i % p.cols);
+    const int64_t zm = i / p.cols;
     const int m = (int)(zm % p.M), z = (int)(zm / p.M);
     if (p.tri && n < m / 128 * 128 / p.nt * p.nt) return;     // tiles left of the diagonal's are not computed
-    if (p.ep_B > 0 && n % p.ep_B >= p.ep_n) return;
     float2 v = p.part[i];
     for (int k = 1; k < p.ksplit; ++k) {
         const float2 w = p.part[(int64_t)k * n_el + i];
@@ -573,12 +584,12 @@ bool aligned2(const void* q, int64_t a, int64_t b, int64_t c) {
 }  // namespace
 
 // Tile widths, the k split and the workspace (float2 elements of `part`).
-// The column tile is the narrowest multiple of 8 that keeps the tile count of
-// 128-wide ones, and the coupling's columns are tiled channel by channel, so
-// that no padding columns beyond 7 are computed (45 beams padded to 128 rows
-// per channel: 3 tiles of 48; 4 sites' coupling and Gram 111 us in whole
-// tiles, 74 us in these).  Callers put the side with few rows on the columns for the same
-// reason: its rows would be padded to 128.  The split: the parts
+// A chunk of a tile takes about 2800 clocks whatever the tile's width (48, 104
+// and 128 columns measured: the cutting warps' chain), so the columns go into
+// as few tiles as they fill; the coupling's columns are taken through all
+// channels without the padding between them (3 channels of 193 beams: 5 tiles
+// where channel by channel takes 6).  Callers put the side with few rows on the
+// columns, since rows are padded to 128.  The split: the parts
 // that minimise rounds x (chunks per part + the pipeline's fill, about three
 // chunks), plus the parts' way through memory at about 2.5 KB per clock.  It
 // is chosen for plan_batch entries, so that a site's sums do not depend on
@@ -590,18 +601,17 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
         o->kper = (o->kvalid + kStep - 1) / kStep * kStep;
         o->vec = o->sk == 1 && aligned2(o->p, o->sr, o->sk2, o->sb);
         if (o->sk != 1 && o->sr != 1) return cudaErrorInvalidValue;
-        // offsets within a tile's chunk are 32-bit in the kernel
-        if (127 * o->sr + kStep > 0x7fffffff || kStep * o->sk > 0x7fffffff) return cudaErrorInvalidValue;
+        // a row's length and offsets within a chunk are 32-bit in the kernel
+        if (o->sr > 0x7fffffff || kStep * o->sk > 0x7fffffff) return cudaErrorInvalidValue;
     }
     if (p.A.kvalid != p.B.kvalid || p.A.nper != p.B.nper) return cudaErrorInvalidValue;
     if (p.dk && p.A.nper != 1) return cudaErrorInvalidValue;
     p.vecC = p.scn == 1 && aligned2(p.C, p.scm, p.scb, 0) ? 1 : 0;
     if (p.ep_B > 0 && (p.ep_n < 1 || p.ep_n > p.ep_B || p.N % p.ep_B)) return cudaErrorInvalidValue;
-    const int cols = p.ep_B > 0 ? p.ep_n : p.N;                // of a channel, or all
-    p.ch_tiles = (cols + 127) / 128;
-    p.nt = ((cols + p.ch_tiles - 1) / p.ch_tiles + 7) / 8 * 8;
-    p.ch_tiles = (cols + p.nt - 1) / p.nt;
-    p.n_tiles = p.ch_tiles * (p.ep_B > 0 ? p.N / p.ep_B : 1);
+    p.cols = p.ep_B > 0 ? p.N / p.ep_B * p.ep_n : p.N;
+    p.n_tiles = (p.cols + 127) / 128;
+    p.nt = ((p.cols + p.n_tiles - 1) / p.n_tiles + 7) / 8 * 8;
+    p.n_tiles = (p.cols + p.nt - 1) / p.nt;
     const int m_tiles = (p.M + 127) / 128;
     p.tiles = 0;
     for (int mt = 0; mt < m_tiles; ++mt) p.tiles += p.n_tiles - (p.tri ? mt * 128 / p.nt : 0);
@@ -610,8 +620,8 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
     const int64_t units = (int64_t)p.tiles * pb;
     if (units * 16 > (1 << 26) || (int64_t)p.tiles * p.batch * 16 > (1 << 26)) return cudaErrorInvalidValue;
     const int sms = num_sms();
-    const double chunk = 12.0 * p.nt;                          // clocks of a chunk's MMAs
-    const double bytes = 8.0 * pb * (double)p.M * p.N;
+    const double chunk = 2800.0;                               // clocks, whatever the width
+    const double bytes = 8.0 * pb * (double)p.M * p.cols;
     double best = 0.0;
     p.ksplit = 1;
     for (int S = 1; S <= 16 && S * 4 <= p.steps; ++S) {
@@ -624,7 +634,7 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
         }
     }
     p.units = p.tiles * p.batch * p.ksplit;
-    *part_elems = p.ksplit > 1 ? (size_t)p.ksplit * p.batch * p.M * p.N : 0;
+    *part_elems = p.ksplit > 1 ? (size_t)p.ksplit * p.batch * p.M * p.cols : 0;
     return cudaSuccess;
 }
 
@@ -637,7 +647,7 @@ cudaError_t bip_cgemm_f32(const CGemmF32& p, cudaStream_t s) {
                   : b      ? launch<false, true>(p, s)
                            : launch<false, false>(p, s);
     if (e != cudaSuccess || p.ksplit == 1) return e;
-    const int64_t n = (int64_t)p.batch * p.M * p.N;
+    const int64_t n = (int64_t)p.batch * p.M * p.cols;
     cgemm_sum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p);
     return cudaGetLastError();
 }
