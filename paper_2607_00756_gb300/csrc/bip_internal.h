@@ -310,7 +310,8 @@ struct CGemmF32 {
     int conjA, conjB;
     const float* dk; int64_t sdb;   // optional real scale of each k (null: 1), with one k block only
     // C(m, n) at C[z scb + m scm + n scn], or with ep_B > 0 (n = (ch, b) = ch
-    // ep_B + b, of which b < ep_n are computed) at C[z scb + b scn + ch ep_Dp + m]
+    // ep_B + b, of which b < ep_n are computed and counted as columns) at
+    // C[z scb + b scn + ch ep_Dp + m]
     float2* C; int64_t scm, scn, scb;
     int ep_B, ep_n, ep_Dp;
     int tri;                        // only the column tiles that reach the diagonal or lie right of it
