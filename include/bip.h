@@ -507,7 +507,9 @@ bip_status bip_build_s1_noalloc(bip_ctx* ctx, const float* V, const bip_atom* at
  *   gives up makes the kernel stop issuing work, let its copies and MMAs in
  *   flight finish (bounded by the built-in limit), free its tensor memory
  *   and set a flag, which the call returns as BIP_ERR_TIMEOUT (capture-safe
- *   contexts: bip_check_errors).  The context stays usable.
+ *   contexts and captured FP32 calls: bip_check_errors).  The flag stays set
+ *   until it is reported, whatever is called or replayed between, and is
+ *   reported once.  The context stays usable.
  * bip_debug_fail_alloc(k): the k-th device allocation the library makes
  *   from now on (in any context) fails as if the device were out of memory,
  *   so that the call returns BIP_ERR_OOM; 0 turns it off.  Resets the count

@@ -977,16 +977,25 @@ void release_map_workspaces(bip_ctx* c, cudaStream_t s) {
         release(*b);
 }
 
-// Waits for the stream and turns the kernels' give-up flag into a status.
-// The flag comes back through pinned memory: a pageable copy waits for the
-// stream and then once more for itself (9 us).  An FP32 context's calls can be
-// captured as they are; there the flag is left to bip_check_errors.
-bip_status check_flag(bip_ctx* c, cudaStream_t s) {
-    if (c->prec == BIP_PREC_FP32 && capturing(s)) return BIP_OK;
+// Waits for the stream and turns the kernels' give-up flag into a status.  The
+// flag is cleared when it is read, never by a launch or at a call's start: the
+// calls that do not read it (capture-safe contexts, captured FP32 calls)
+// leave it for bip_check_errors, and what runs between would wipe it.
+// It comes back through pinned memory: a pageable copy waits for the stream and
+// then once more for itself (9 us).
+bip_status read_flag(bip_ctx* c, cudaStream_t s) {
     CUDA_TRY(c, cudaMemcpyAsync(c->flag_h, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(c, cudaStreamSynchronize(s));
-    if (*c->flag_h) return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
-    return BIP_OK;
+    if (!*c->flag_h) return BIP_OK;
+    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
+    return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
+}
+
+// ... at a call's end.  An FP32 context's calls can be captured as they are;
+// there the flag is left to bip_check_errors.
+bip_status check_flag(bip_ctx* c, cudaStream_t s) {
+    if (c->prec == BIP_PREC_FP32 && capturing(s)) return BIP_OK;
+    return read_flag(c, s);
 }
 
 // One FP32 contraction of cgemm_f32.cu: its plan, the workspace of a split k
@@ -1767,7 +1776,6 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
             CUDA_TRY(c, ensure(c->ybuf, SB * 2 * P64r * nch * K * sizeof(uint16_t), true, s));
         }
     }
-    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     CUDA_TRY(c, ensure(c->q32, SB * perQ * sizeof(float2), true, s));
     // G(Delta) of every site when the raster evaluation runs once at the end,
     // else of one batch
@@ -2390,7 +2398,6 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
     CUDA_TRY(c, ensure(c->xopA, SB * perA * 8, true, s));
     CUDA_TRY(c, ensure(c->xopB, SB * perB * 8, true, s));
     CUDA_TRY(c, ensure(c->xm32, SB * perMt * sizeof(float2), true, s));
-    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
 
     // On a raster scan list the per-beam contraction separates over the
     // aperture beams' lattice (cube_raster.cu)
@@ -2756,7 +2763,6 @@ bip_status bip_debug_cgemm(bip_ctx* c, int32_t M, int32_t N, int32_t K, int32_t 
     cudaStream_t s = (cudaStream_t)stream;
     bip_status st = make_tables(c, s);
     if (st != BIP_OK) return st;
-    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     CGemmF32 p{};
     p.M = M; p.N = N; p.batch = batch;
     p.A = CGemmOperand{(const float2*)A, sA[0], sA[1], sA[2], K, blocks, sA[3], 0, 0};
@@ -2845,16 +2851,8 @@ bip_status bip_set_capture_safe(bip_ctx* c, int32_t on) {
 
 bip_status bip_check_errors(bip_ctx* c, void* stream) {
     if (!c) return BIP_ERR_INVALID_ARG;
-    if (!c->errflag.p) return BIP_OK;
-    cudaStream_t s = (cudaStream_t)stream;
-    int flag = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(&flag, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(c, cudaStreamSynchronize(s));
-    if (flag) {
-        CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
-        return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
-    }
-    return BIP_OK;
+    if (!c->errflag.p || !c->flag_h) return BIP_OK;
+    return read_flag(c, (cudaStream_t)stream);
 }
 
 bip_status bip_set_raster_eval(bip_ctx* c, int32_t on) {
@@ -3107,7 +3105,6 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
             CUDA_TRY(c, ensure(c->g_sB2, SB * 4 * (size_t)K * KB * sizeof(uint16_t), true, s));
         }
     }
-    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     CUDA_TRY(c, ensure(c->opA32, SB * perA * sizeof(float2), true, s));
     CUDA_TRY(c, ensure(c->opB32, SB * perB * sizeof(float2), true, s));
     st = operand_layout(c, K, s);
@@ -3611,7 +3608,6 @@ bip_status bip_site_coupling(bip_ctx* c, const void* H, int32_t site, void* m_ou
         g2.out_c64 = (float2*)opA.p; g2.site_stride = (int64_t)perA;
         g1.out_c64 = (float2*)opB.p; g1.site_stride = (int64_t)perB;
     }
-    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
     if (f8) {
         bip_status st = f8_hmax(c, H, s);
         if (st != BIP_OK) return st;
