@@ -55,7 +55,8 @@ typedef enum {
     BIP_ERR_SHAPE = 2,         /* sizes inconsistent with the configuration   */
     BIP_ERR_OOM = 3,           /* a device or host allocation failed          */
     BIP_ERR_CUDA = 4,          /* a CUDA call failed (text in bip_last_error) */
-    BIP_ERR_TIMEOUT = 5,       /* a device-side wait gave up                  */
+    BIP_ERR_TIMEOUT = 5,       /* a device-side wait gave up (FP32: in this call
+                                  or one before it, see bip_set_wait_limit)   */
     BIP_ERR_UNSUPPORTED = 6,   /* valid request the library does not implement */
     BIP_ERR_NUMERIC = 7        /* an output holds NaN or Inf (only with
                                   bip_set_check_finite on)                    */
@@ -506,10 +507,16 @@ bip_status bip_build_s1_noalloc(bip_ctx* ctx, const float* V, const bip_atom* at
  *   tensor-core kernels of this context (0: the built-in 4 s).  A wait that
  *   gives up makes the kernel stop issuing work, let its copies and MMAs in
  *   flight finish (bounded by the built-in limit), free its tensor memory
- *   and set a flag, which the call returns as BIP_ERR_TIMEOUT (capture-safe
- *   contexts and captured FP32 calls: bip_check_errors).  The flag stays set
- *   until it is reported, whatever is called or replayed between, and is
- *   reported once.  The context stays usable.
+ *   and set a flag.  In the tensor-core precisions the call waits for its
+ *   launches and returns it as BIP_ERR_TIMEOUT (capture-safe contexts:
+ *   bip_check_errors).  FP32 calls return with their work queued; theirs is
+ *   reported by whatever comes first of the next call on the context (which
+ *   then does nothing else), bip_check_errors, and a wait the call itself
+ *   makes for a host result (the aberration derivatives, the finite check,
+ *   the autotuner); capture-safe contexts and captured calls:
+ *   bip_check_errors.  The flag stays set until it is reported, whatever is
+ *   called or replayed between, and is reported once.  The context stays
+ *   usable.
  * bip_debug_fail_alloc(k): the k-th device allocation the library makes
  *   from now on (in any context) fails as if the device were out of memory,
  *   so that the call returns BIP_ERR_OOM; 0 turns it off.  Resets the count

@@ -21,6 +21,7 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr int kRowPad = 128;        // aperture-side operand rows: the MMA's 128-row tiles
 constexpr int kDetPad = 32;         // detector-side rows: the N of a tile (multiple of 16, K of the Gram a multiple of 32)
 constexpr int kScanTile = 256;      // scans per quadratic-form work item
+constexpr int kFlag32 = 8;          // an FP32 context's give-up flag in bip_ctx::flag_h
 constexpr int kProbeMaxScans = 2048; // the probe order keeps Psi of every scan for a batch of sites
 
 struct DevBuf {
@@ -109,8 +110,11 @@ struct bip_ctx {
     DevBuf aw1[6], aw2[6];              // per-target / per-parent weights (reconstruction adjoint)
     bool adj_tables = false;
     DevBuf f8pmax, f8inv0, f8inv1, f8hmax, f8H, f8sA, f8sB;   // FP8 per-window scales
-    DevBuf errflag;
-    int* flag_h = nullptr;              // pinned copy of the flag
+    DevBuf errflag;                     // give-up flag of the tensor-core precisions' kernels
+    // pinned: [0] the copy errflag is read through, [kFlag32] the flag of an
+    // FP32 context's contractions, which write it there themselves
+    int* flag_h = nullptr;
+    cudaEvent_t ev_flag = nullptr;      // the end of the last FP32 call
     std::vector<int32_t> work_h;
     bool check_finite = false;          // scan outputs for NaN / Inf (bip_set_check_finite)
     DevBuf nf_count;
@@ -492,7 +496,11 @@ bip_status make_tables(bip_ctx* c, cudaStream_t s) {
     CUDA_TRY(c, upload(c->hcube, hc, s));
     CUDA_TRY(c, upload(c->shcube, shc, s));
     CUDA_TRY(c, ensure(c->errflag, 64, true, s));
-    if (!c->flag_h) CUDA_TRY(c, cudaMallocHost((void**)&c->flag_h, 64));
+    if (!c->flag_h) {
+        CUDA_TRY(c, cudaMallocHost((void**)&c->flag_h, 64));
+        std::memset(c->flag_h, 0, 64);
+    }
+    if (!c->ev_flag) CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_flag, cudaEventDisableTiming));
     c->tables = true;
     return BIP_OK;
 }
@@ -838,6 +846,7 @@ bip_status bip_destroy(bip_ctx* c) {
                      &c->cr_ay, &c->cr_ax, &c->cr_cy, &c->cr_cx, &c->cr_T, &c->nf_count, &c->twhw, &c->cols2, &c->gpart};
     for (DevBuf* b : all) release(*b);
     if (c->flag_h) cudaFreeHost(c->flag_h);
+    if (c->ev_flag) cudaEventDestroy(c->ev_flag);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->side) cudaStreamDestroy(c->side);
@@ -977,25 +986,49 @@ void release_map_workspaces(bip_ctx* c, cudaStream_t s) {
         release(*b);
 }
 
-// Waits for the stream and turns the kernels' give-up flag into a status.  The
-// flag is cleared when it is read, never by a launch or at a call's start: the
-// calls that do not read it (capture-safe contexts, captured FP32 calls)
-// leave it for bip_check_errors, and what runs between would wipe it.
-// It comes back through pinned memory: a pageable copy waits for the stream and
-// then once more for itself (9 us).
-bip_status read_flag(bip_ctx* c, cudaStream_t s) {
-    CUDA_TRY(c, cudaMemcpyAsync(c->flag_h, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(c, cudaStreamSynchronize(s));
-    if (!*c->flag_h) return BIP_OK;
-    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
+bip_status gave_up(bip_ctx* c) {
     return fail(c, BIP_ERR_TIMEOUT, "a tensor-core contraction gave up waiting (device timeout)");
 }
 
-// ... at a call's end.  An FP32 context's calls can be captured as they are;
-// there the flag is left to bip_check_errors.
+// The give-up flag of FP32 contractions whose stream has been waited for.
+bip_status flag32(bip_ctx* c) {
+    volatile int* f = c->flag_h + kFlag32;
+    if (!*f) return BIP_OK;
+    *f = 0;
+    return gave_up(c);
+}
+
+// Waits for the stream and turns the kernels' give-up flags into a status.  A
+// flag is cleared when it is read, never by a launch or at a call's start: the
+// calls that do not read it (capture-safe contexts, FP32 calls) leave it, and
+// what runs between would wipe it.  errflag comes back through pinned memory:
+// a pageable copy waits for the stream and then once more for itself (9 us).
+bip_status read_flag(bip_ctx* c, cudaStream_t s) {
+    CUDA_TRY(c, cudaMemcpyAsync(c->flag_h, c->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(c, cudaStreamSynchronize(s));
+    const bip_status st = flag32(c);
+    if (!*c->flag_h) return st;
+    CUDA_TRY(c, cudaMemsetAsync(c->errflag.p, 0, sizeof(int), s));
+    return gave_up(c);
+}
+
+// At a call's end.  An FP32 call returns with its work queued: the next call
+// (earlier_give_up), bip_check_errors or a wait the call makes for another
+// result reports its flag, and a program that drives several contexts from
+// one thread keeps their overlap.
 bip_status check_flag(bip_ctx* c, cudaStream_t s) {
-    if (c->prec == BIP_PREC_FP32 && capturing(s)) return BIP_OK;
-    return read_flag(c, s);
+    if (c->prec != BIP_PREC_FP32) return read_flag(c, s);
+    if (!capturing(s)) CUDA_TRY(c, cudaEventRecord(c->ev_flag, s));
+    return BIP_OK;
+}
+
+// At a call's start: whether a contraction of an earlier FP32 call has given
+// up (capture-safe contexts leave that to bip_check_errors).
+bip_status earlier_give_up(bip_ctx* c, cudaStream_t s) {
+    if (!c->flag_h || c->capture_safe || !*(volatile int*)(c->flag_h + kFlag32) || capturing(s)) return BIP_OK;
+    CUDA_TRY(c, cudaEventSynchronize(c->ev_flag));     // its other blocks have set the flag too
+    flag32(c);
+    return fail(c, BIP_ERR_TIMEOUT, "a contraction of an earlier call gave up waiting (device timeout)");
 }
 
 // One FP32 contraction of cgemm_f32.cu: its plan, the workspace of a split k
@@ -1010,7 +1043,7 @@ cudaError_t cgemm(bip_ctx* c, CGemmF32 p, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     p.part = (float2*)c->gpart.p;
-    p.err = (int*)c->errflag.p;
+    p.err = c->prec == BIP_PREC_FP32 ? c->flag_h + kFlag32 : (int*)c->errflag.p;
     p.wait_ns = c->wait_ns;
     return bip_cgemm_f32(p, s);
 }
@@ -2673,6 +2706,10 @@ bip_status finite_check(bip_ctx* c, std::initializer_list<OutSpan> spans, cudaSt
     unsigned long long bad = 0;
     CUDA_TRY(c, cudaMemcpyAsync(&bad, c->nf_count.p, sizeof(bad), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(c, cudaStreamSynchronize(s));
+    if (!c->capture_safe) {
+        const bip_status st = flag32(c);
+        if (st != BIP_OK) return st;
+    }
     if (bad) return fail(c, BIP_ERR_NUMERIC, std::to_string(bad) + " output values are NaN or infinite");
     return BIP_OK;
 }
@@ -2692,6 +2729,7 @@ bip_status bip_coreloss_map(bip_ctx* c, const void* H, const double* scan_px, in
     BIP_RANGE("bip_coreloss_map");
     bip_status st = check_map_args(c, H, scan_px, P, map_out);
     if (st == BIP_OK) st = refuse_check_under_capture(c, (cudaStream_t)stream);
+    if (st == BIP_OK) st = earlier_give_up(c, (cudaStream_t)stream);
     if (st != BIP_OK) return st;
     st = run_map(c, H, scan_px, P, nullptr, map_out, nullptr, (cudaStream_t)stream);
     if (st != BIP_OK) return st;
@@ -2703,6 +2741,7 @@ bip_status bip_coreloss_sites(bip_ctx* c, const void* H, const double* scan_px, 
     BIP_RANGE("bip_coreloss_sites");
     bip_status st = check_map_args(c, H, scan_px, P, partial_out);
     if (st == BIP_OK) st = refuse_check_under_capture(c, (cudaStream_t)stream);
+    if (st == BIP_OK) st = earlier_give_up(c, (cudaStream_t)stream);
     if (st != BIP_OK) return st;
     st = run_map(c, H, scan_px, P, partial_out, nullptr, nullptr, (cudaStream_t)stream);
     if (st != BIP_OK) return st;
@@ -2721,6 +2760,7 @@ bip_status bip_coreloss_cube(bip_ctx* c, const float* V, const void* H, const do
     for (int i = 0; i < 2 * P; ++i)
         if (!std::isfinite(scan_px[i])) return fail(c, BIP_ERR_INVALID_ARG, "scan position is not finite");
     bip_status st = refuse_check_under_capture(c, (cudaStream_t)stream);
+    if (st == BIP_OK) st = earlier_give_up(c, (cudaStream_t)stream);
     if (st != BIP_OK) return st;
     st = run_cube_exact(c, V, H, scan_px, P, cube_out, (cudaStream_t)stream);
     if (st != BIP_OK) return st;
@@ -2775,7 +2815,7 @@ bip_status bip_debug_cgemm(bip_ctx* c, int32_t M, int32_t N, int32_t K, int32_t 
         p.scn = M;
     }
     CUDA_TRY(c, cgemm(c, p, s));
-    return check_flag(c, s);
+    return read_flag(c, s);
 }
 
 bip_status bip_debug_split(bip_ctx* c, int32_t rows, int32_t cols, const void* src, int64_t s_row, int64_t s_col,
@@ -2831,6 +2871,7 @@ bip_status bip_coreloss_qeels(bip_ctx* c, const void* H, const double* scan_px, 
                     "or dfx = 1 (axis 1)");
     cudaStream_t s = (cudaStream_t)stream;
     st = refuse_check_under_capture(c, s);
+    if (st == BIP_OK) st = earlier_give_up(c, s);
     if (st != BIP_OK) return st;
     CUDA_TRY(c, ensure(c->cube_scratch, (size_t)P * c->geo.n_det * sizeof(float), false, s));
     CUDA_TRY(c, upload(c->bin_of_d, bin_of, s));
@@ -2886,6 +2927,8 @@ bip_status bip_autotune(bip_ctx* c, const void* H, const double* scan_px, int32_
     bip_status st = check_map_args(c, H, scan_px, P, map_out);
     if (st != BIP_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
+    st = earlier_give_up(c, s);
+    if (st != BIP_OK) return st;
     const bool tc = c->prec != BIP_PREC_FP32;
     cudaEvent_t e0, e1;
     CUDA_TRY(c, cudaEventCreate(&e0));
@@ -2904,6 +2947,8 @@ bip_status bip_autotune(bip_ctx* c, const void* H, const double* scan_px, int32_
         if (r != BIP_OK) return r;
         CUDA_TRY(c, cudaEventRecord(e1, s));
         CUDA_TRY(c, cudaEventSynchronize(e1));
+        r = flag32(c);
+        if (r != BIP_OK) return r;
         float t = 0.f;
         CUDA_TRY(c, cudaEventElapsedTime(&t, e0, e1));
         *ms = t / 2.0;
@@ -3053,6 +3098,8 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
     if (d_V && !V) return fail(c, BIP_ERR_INVALID_ARG, "d_V needs the V the matrices were built from");
     if ((reinterpret_cast<uintptr_t>(d_H) & 7) != 0) return fail(c, BIP_ERR_INVALID_ARG, "d_H must be 8-byte aligned");
     cudaStream_t s = (cudaStream_t)stream;
+    st = earlier_give_up(c, s);
+    if (st != BIP_OK) return st;
     const bip_config& g = c->cfg;
     const BipGeometry& geo = c->geo;
     const int K = g.win * g.win, Bpad = c->Bpad, Dpad = c->Dpad, nch = c->nch_max, B = geo.B;
@@ -3407,6 +3454,8 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
         std::vector<double2> D(B);
         CUDA_TRY(c, cudaMemcpyAsync(D.data(), c->g_Dsum.p, (size_t)B * sizeof(double2), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(c, cudaStreamSynchronize(s));
+        st = flag32(c);
+        if (st != BIP_OK) return st;
         // dL/dtheta = -2 sum_b chi'_b Im D_b
         double gdf = 0.0, gcs = 0.0;
         for (int b = 0; b < B; ++b) {
@@ -3579,6 +3628,8 @@ bip_status bip_site_coupling(bip_ctx* c, const void* H, int32_t site, void* m_ou
     if (site < 0 || site >= c->n_sites) return fail(c, BIP_ERR_INVALID_ARG, "site out of range");
     if (c->uneven) return fail(c, BIP_ERR_UNSUPPORTED, "the site coupling is given at the context's window only");
     cudaStream_t s = (cudaStream_t)stream;
+    const bip_status earlier = earlier_give_up(c, s);
+    if (earlier != BIP_OK) return earlier;
     const bip_config& g = c->cfg;
     const BipGeometry& geo = c->geo;
     const int K = g.win * g.win, Bpad = c->Bpad, Dpad = c->Dpad, nch = c->nch_max;

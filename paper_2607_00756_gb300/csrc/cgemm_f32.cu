@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_f32_kernel(const __grid_con
 
     auto fail = [&]() {
         *abort_flag = 1;
-        atomicExch(p.err, 1);
+        *(volatile int*)p.err = 1;               // device memory, or pinned host memory
     };
 
     // lane 0 waits for its warp

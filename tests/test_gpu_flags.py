@@ -94,3 +94,66 @@ def test_flag_outlives_the_next_call_of_a_graph(env):
         assert right(ctx, env)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("report", ["next call", "check_errors", "finite check", "aberrations"])
+def test_fp32_give_up_is_reported(env, report):
+    """An FP32 call does not wait for its launches: a wait of theirs that ran
+    out is reported by the next call on the context, by bip_check_errors, or
+    by the call itself where it waits for a result; once, and the context
+    stays usable."""
+    capi, make, sp, want, V, H = env
+    ctx = make("fp32")
+    try:
+        assert right(ctx, env)
+        capi.bip_set_wait_limit(ctx.ctx, 1)
+        if report == "finite check":
+            ctx.set_check_finite(1)
+            timeout(capi, lambda: ctx.map(H, sp.scans))
+            ctx.set_check_finite(0)
+        elif report == "aberrations":
+            g = torch.ones(len(sp.scans), dtype=torch.float64, device="cuda")
+            timeout(capi, lambda: ctx.grad(H, sp.scans, g, occ=False, h=False))
+        else:
+            ctx.map(H, sp.scans)
+            torch.cuda.synchronize()
+        capi.bip_set_wait_limit(ctx.ctx, 0)
+        if report == "next call":
+            timeout(capi, lambda: ctx.map(H, sp.scans))
+        elif report == "check_errors":
+            timeout(capi, lambda: capi.bip_check_errors(ctx.ctx))
+        capi.bip_check_errors(ctx.ctx)
+        assert right(ctx, env)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("name", ["map", "sites", "coupling", "grad", "cube", "qeels"])
+def test_fp32_calls_return_with_their_work_queued(env, name):
+    """Behind 0.2 s of other work on the stream a warmed-up call returns
+    before that work is done."""
+    from paper_2607_00756_gb300.context import BipContext
+    capi, make, sp, want, V, H = env
+    g = torch.ones(len(sp.scans), dtype=torch.float64, device="cuda")
+    ctx = make("fp32")
+    if name == "qeels":
+        ctx.close()
+        ctx = BipContext(synth.config1().replace(dfy=1), prec="fp32")
+        ctx.build(V, sp.atoms, sp.nch)
+    call = {"map": lambda: ctx.map(H, sp.scans), "sites": lambda: ctx.sites(H, sp.scans), "coupling": lambda: ctx.coupling(H, 0),
+            "grad": lambda: ctx.grad(H, sp.scans, g, occ=True, aberr=False, V=V)["H"], "cube": lambda: ctx.cube(V, H, sp.scans),
+            "qeels": lambda: ctx.qeels(H, sp.scans, 0)[1]}[name]
+    try:
+        a = call()
+        torch.cuda.synchronize()
+        torch.cuda._sleep(400_000_000)
+        b = call()
+        done = torch.cuda.Event()
+        done.record()
+        assert not done.query()
+        torch.cuda.synchronize()
+        a, b = (torch.view_as_real(t) if t.is_complex() else t for t in (a, b))
+        assert torch.equal(a, b)
+        capi.bip_check_errors(ctx.ctx)
+    finally:
+        ctx.close()
