@@ -237,7 +237,8 @@ bip_status bip_build(bip_ctx* ctx, const float* V, const bip_atom* atoms, int32_
  *            bip_set_site_windows: [sum_sites nch w^2] in all); 16-byte
  *            aligned (else BIP_ERR_INVALID_ARG).
  *   scan_px  [P, 2] float64 host: scan positions in pixels (y, x).
- *   map_out  [P] float64 device.
+ *   map_out  [P] float64 device; as it was when the call returns
+ *            BIP_ERR_TIMEOUT.
  * Requires both builds on this context (else BIP_ERR_INVALID_ARG). */
 bip_status bip_coreloss_map(bip_ctx* ctx, const void* H, const double* scan_px,
                             int32_t P, double* map_out, void* stream);

@@ -2291,11 +2291,14 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
         d.partial = partial;
         TIMED(c, BIP_STAGE_QUADFORM, s, bip_raster_eval(d, rargs, s));
     }
-    // the site sum goes out before the wait for the flag
+    // the site sum goes out before the wait for the flag, and reads the flag
+    // itself where the call is going to return it: such a call has not
+    // written its map
     if (map_out && !cube_out) {
         CUDA_TRY(c, ensure(c->rsum, bip_reduce_scratch_bytes(c->n_sites, P), false, s));
         const double* occ = c->occ_n == c->n_sites ? (const double*)c->occ_d.p : nullptr;
-        TIMED(c, BIP_STAGE_REDUCE, s, bip_reduce_sites(partial, c->n_sites, P, c->rsum.p, map_out, s, occ));
+        const int* gave_up = tc && !c->capture_safe ? (const int*)c->errflag.p : nullptr;
+        TIMED(c, BIP_STAGE_REDUCE, s, bip_reduce_sites(partial, c->n_sites, P, c->rsum.p, map_out, s, occ, gave_up));
         if (c->n_sites > 0) c->launches[BIP_STAGE_REDUCE]++;   // two kernels: chunks, then their sum
     }
     if (!c->capture_safe) {

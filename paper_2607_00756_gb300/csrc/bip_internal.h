@@ -381,9 +381,10 @@ size_t bip_reduce_scratch_bytes(int n_sites, int P);
 // adds to *count the NaN or infinite values among n values of elem_bytes (4: float, 8: double)
 cudaError_t bip_count_nonfinite(const void* v, int64_t n, int elem_bytes, unsigned long long* count, cudaStream_t s);
 // occ (optional, [n_sites]): each site's contribution is weighted by its
-// occupancy before the sum
+// occupancy before the sum; gave_up (optional, device): map_out is not written
+// when it is set by then
 cudaError_t bip_reduce_sites(const float* partial, int n_sites, int P, void* scratch, double* map_out,
-                             cudaStream_t s, const double* occ = nullptr);
+                             cudaStream_t s, const double* occ = nullptr, const int* gave_up = nullptr);
 
 // gemm_tc.cu : tcgen05 complex contractions in split BF16 or BF16.
 // Operands are bf16 planes, K contiguous -- four (re_hi, re_lo, im_hi,

@@ -38,10 +38,13 @@ __global__ void __launch_bounds__(kThreads) reduce_chunk_kernel(const float* __r
     chunk_sum[(size_t)blockIdx.y * P + p] = make_double2(s, c);
 }
 
+// gave_up (nullable): the flag of the contractions before; once set, out stays
+// as it is
 __global__ void __launch_bounds__(kThreads) reduce_final_kernel(const double2* __restrict__ chunk_sum, int n_chunks,
-                                                                int P, double* __restrict__ out) {
+                                                                int P, double* __restrict__ out,
+                                                                const int* __restrict__ gave_up) {
     const int p = blockIdx.x * kThreads + threadIdx.x;
-    if (p >= P) return;
+    if (p >= P || (gave_up && *gave_up)) return;
     double s = 0.0, c = 0.0;
     for (int j = 0; j < n_chunks; ++j) {
         const double2 v = chunk_sum[(size_t)j * P + p];
@@ -58,7 +61,7 @@ size_t bip_reduce_scratch_bytes(int n_sites, int P) {
 }
 
 cudaError_t bip_reduce_sites(const float* partial, int n_sites, int P, void* scratch, double* out, cudaStream_t s,
-                             const double* occ) {
+                             const double* occ, const int* gave_up) {
     const int n_chunks = (n_sites + kChunk - 1) / kChunk;
     if (n_chunks == 0) return cudaMemsetAsync(out, 0, (size_t)P * sizeof(double), s);
     double2* cs = static_cast<double2*>(scratch);
@@ -66,7 +69,7 @@ cudaError_t bip_reduce_sites(const float* partial, int n_sites, int P, void* scr
                                                                                          cs);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    reduce_final_kernel<<<(P + kThreads - 1) / kThreads, kThreads, 0, s>>>(cs, n_chunks, P, out);
+    reduce_final_kernel<<<(P + kThreads - 1) / kThreads, kThreads, 0, s>>>(cs, n_chunks, P, out, gave_up);
     return cudaGetLastError();
 }
 

@@ -157,3 +157,18 @@ def test_fp32_calls_return_with_their_work_queued(env, name):
         capi.bip_check_errors(ctx.ctx)
     finally:
         ctx.close()
+
+
+def test_map_that_gave_up_leaves_its_output(env):
+    """A map that returns BIP_ERR_TIMEOUT has not written map_out."""
+    capi, make, sp, want, V, H = env
+    ctx = make("mixed")
+    try:
+        out = torch.full((len(sp.scans),), 7.0, dtype=torch.float64, device="cuda")
+        capi.bip_set_wait_limit(ctx.ctx, 1)
+        timeout(capi, lambda: ctx.map(H, sp.scans, out=out))
+        assert torch.all(out == 7.0)
+        capi.bip_set_wait_limit(ctx.ctx, 0)
+        assert right(ctx, env)
+    finally:
+        ctx.close()
