@@ -395,7 +395,9 @@ bip_status bip_set_site_windows(bip_ctx* ctx, const int32_t* win, void* stream);
  * sum_tau (Q_tau R_tau)_bb -- the contractions in FP32 on every precision;
  * d_occ uses the context's precision for I_tau.
  *   dL_dI [P] float64 device; other requirements as bip_coreloss_map;
- *   d_H 8-byte aligned.  Synchronises the stream when d_aberr is given. */
+ *   d_H 8-byte aligned.  Synchronises the stream when d_aberr is given.
+ * An FP32 call without d_aberr can be captured after one like it; its scan
+ * list is then copied into the context, which keeps it for the replays. */
 bip_status bip_coreloss_grad(bip_ctx* ctx, const float* V, const void* H, const double* scan_px,
                              int32_t P, const double* dL_dI, double* d_occ, void* d_H,
                              double* d_aberr, float* d_V, void* stream);

@@ -81,6 +81,8 @@ struct bip_ctx {
     DevBuf occ_d;                       // site occupancies weighting the site sum
     int occ_n = 0;                      // sites they were given for (0: none)
     DevBuf g_s1, g_w, g_R, g_gmt, g_T, g_D, g_Dsum;   // gradient pass workspaces
+    DevBuf g_scans;                     // its scan list: scans_d is the maps', which may keep theirs
+    std::vector<std::vector<double>> captured_scans;   // host lists that captured gradients copy from
     DevBuf g_s1bar, g_s2bar, g_ubar, g_dA, g_dt1, g_dt2, g_dV2;
     DevBuf g_adj[2], g_ckpt[2], g_seg[2], g_gvp[2];   // of the two adjoint sweeps, which run side by side
     DevBuf gpart;                       // parts of a split k range (cgemm_f32.cu)
@@ -836,7 +838,7 @@ bip_status bip_destroy(bip_ctx* c) {
                      &c->gdiff, &c->kb_d, &c->lat_d, &c->work_d, &c->partial, &c->opA32, &c->opB32, &c->mt32, &c->q32, &c->opA16,
                      &c->opB16, &c->mt16, &c->q16, &c->errflag, &c->rsum, &c->wtc, &c->xtc, &c->illum,
                      &c->cube_scratch, &c->bin_of_d, &c->op8A, &c->op8B, &c->f8pmax, &c->f8inv0, &c->f8inv1,
-                     &c->f8hmax, &c->f8H, &c->f8sA, &c->f8sB, &c->occ_d, &c->g_s1, &c->g_w, &c->g_R,
+                     &c->f8hmax, &c->f8H, &c->f8sA, &c->f8sB, &c->occ_d, &c->g_s1, &c->g_w, &c->g_R, &c->g_scans,
                      &c->g_gmt, &c->g_T, &c->g_D, &c->g_Dsum, &c->g_s1bar, &c->g_s2bar, &c->g_ubar, &c->g_dA,
                      &c->g_dt1, &c->g_dt2, &c->g_dV2, &c->g_adj[0], &c->g_ckpt[0], &c->g_seg[0], &c->g_gvp[0],
                      &c->g_adj[1], &c->g_ckpt[1], &c->g_seg[1], &c->g_gvp[1], &c->pyc, &c->pxc,
@@ -3093,6 +3095,15 @@ bip_status bip_set_aberrations(bip_ctx* c, double defocus, double cs, void* stre
     return BIP_OK;
 }
 
+// The context's own copy of a scan list for a graph to copy from at every
+// replay, when the caller's may be gone; one copy per list, until bip_destroy.
+static const double* kept_scans(bip_ctx* c, const double* scans, int P) {
+    for (const auto& v : c->captured_scans)
+        if (v.size() == (size_t)P * 2 && std::equal(v.begin(), v.end(), scans)) return v.data();
+    c->captured_scans.emplace_back(scans, scans + 2 * (size_t)P);
+    return c->captured_scans.back().data();
+}
+
 static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const double* scan_px, int32_t P,
                                 const double* dL_dI, double* d_occ, void* d_H, double* d_aberr, float* d_V,
                                 void* stream) {
@@ -3129,10 +3140,11 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
     }
     // FP32 contraction per batch of sites: S2, H_n S1 and S1 windows, M (as
     // Mt[b][(n, d)]), Q, then the reverse steps
-    CUDA_TRY(c, ensure(c->scans_d, (size_t)P * 2 * sizeof(double), false, s));
-    CUDA_TRY(c, cudaMemcpyAsync(c->scans_d.p, scan_px, (size_t)P * 2 * sizeof(double), cudaMemcpyHostToDevice, s));
+    CUDA_TRY(c, ensure(c->g_scans, (size_t)P * 2 * sizeof(double), false, s));
+    CUDA_TRY(c, cudaMemcpyAsync(c->g_scans.p, capturing(s) ? kept_scans(c, scan_px, P) : scan_px,
+                                (size_t)P * 2 * sizeof(double), cudaMemcpyHostToDevice, s));
     CUDA_TRY(c, ensure(c->illum, (size_t)Bpad * P * sizeof(float2), false, s));
-    IllumArgs ia{P, B, Bpad, (const int2*)c->hbeam.p, (const double2*)c->coef.p, (const double*)c->scans_d.p, g.ny,
+    IllumArgs ia{P, B, Bpad, (const int2*)c->hbeam.p, (const double2*)c->coef.p, (const double*)c->g_scans.p, g.ny,
                  g.nx, (float2*)c->illum.p};
     CUDA_TRY(c, bip_illum(ia, s));
     const int SB = std::min(c->n_sites, 8);
@@ -3178,7 +3190,7 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
     }
     GradArgs ga{};
     ga.P = P; ga.K = K; ga.B = B;
-    ga.scans = (const double*)c->scans_d.p;
+    ga.scans = (const double*)c->g_scans.p;
     ga.dL_dI = dL_dI;
     ga.occ = occ;
     ga.sites = (const SiteDev*)c->sites_d.p;
