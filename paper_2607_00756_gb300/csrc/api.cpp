@@ -86,6 +86,7 @@ struct bip_ctx {
     DevBuf g_s1bar, g_s2bar, g_ubar, g_dA, g_dt1, g_dt2, g_dV2;
     DevBuf g_adj[2], g_ckpt[2], g_seg[2], g_gvp[2];   // of the two adjoint sweeps, which run side by side
     DevBuf gpart;                       // parts of a split k range (cgemm_f32.cu)
+    std::vector<DevBuf> gpart_old;      // ... outgrown
     DevBuf g_tA, g_tB, g_sA2, g_sB2;    // split-BF16 operands of the reverse-pass contractions
     DevBuf cubeA, cubeB, cube_work, cube_mask;   // the cube on tcgen05
     DevBuf cube_grp, cube_wmap, mpart;  // cube-mode work groups; map modes' item map and column sums
@@ -847,6 +848,7 @@ bip_status bip_destroy(bip_ctx* c) {
                      &c->hcube, &c->shcube, &c->cstash, &c->ccols, &c->xopA, &c->xopB, &c->xm32, &c->tcache,
                      &c->cr_ay, &c->cr_ax, &c->cr_cy, &c->cr_cx, &c->cr_T, &c->nf_count, &c->twhw, &c->cols2, &c->gpart};
     for (DevBuf* b : all) release(*b);
+    for (DevBuf& b : c->gpart_old) release(b);
     if (c->flag_h) cudaFreeHost(c->flag_h);
     if (c->ev_flag) cudaEventDestroy(c->ev_flag);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -986,6 +988,8 @@ void release_map_workspaces(bip_ctx* c, cudaStream_t s) {
                       &c->s1t, &c->psi, &c->ybuf, &c->xtc, &c->f8pmax, &c->f8inv0, &c->f8inv1, &c->f8sA,
                       &c->f8sB})
         release(*b);
+    for (DevBuf& b : c->gpart_old) release(b);
+    c->gpart_old.clear();
 }
 
 bip_status gave_up(bip_ctx* c) {
@@ -1033,6 +1037,21 @@ bip_status earlier_give_up(bip_ctx* c, cudaStream_t s) {
     return fail(c, BIP_ERR_TIMEOUT, "a contraction of an earlier call gave up waiting (device timeout)");
 }
 
+// The workspace of a split k range, one for every FP32 contraction of the
+// context, whose sizes differ: a gradient or a cube may need more than the map
+// that a graph holds and writes here at each replay.  So an outgrown block is
+// kept (the sizes come from the context's few shapes, 10 to 100 MB each), which
+// also spares the wait for the stream before a block could be freed.
+cudaError_t part_buffer(bip_ctx* c, size_t bytes, cudaStream_t s) {
+    if (c->gpart.cap >= bytes) return cudaSuccess;
+    DevBuf larger;
+    const cudaError_t e = ensure(larger, bytes, false, s);
+    if (e != cudaSuccess) return e;
+    if (c->gpart.p) c->gpart_old.push_back(c->gpart);
+    c->gpart = larger;
+    return cudaSuccess;
+}
+
 // One FP32 contraction of cgemm_f32.cu: its plan, the workspace of a split k
 // range, the launch.
 cudaError_t cgemm(bip_ctx* c, CGemmF32 p, cudaStream_t s) {
@@ -1041,7 +1060,7 @@ cudaError_t cgemm(bip_ctx* c, CGemmF32 p, cudaStream_t s) {
     cudaError_t e = bip_cgemm_plan(p, &part);
     if (e != cudaSuccess) return e;
     if (part > 0) {
-        e = ensure(c->gpart, part * sizeof(float2), false, s);
+        e = part_buffer(c, part * sizeof(float2), s);
         if (e != cudaSuccess) return e;
     }
     p.part = (float2*)c->gpart.p;
