@@ -1305,35 +1305,50 @@ int isqrt_up(int n) {
     return k;
 }
 
-// Workspaces `set` of an adjoint sweep over n slices of ncol columns, its
-// checkpoints every ceil(sqrt(n)) slices.
-bip_status adjoint_alloc(bip_ctx* c, int set, int ncol, int n, cudaStream_t s) {
-    const size_t G = (size_t)c->cfg.ny * c->cfg.nx, state = (size_t)ncol * G;
+// Workspaces of an adjoint sweep over n slices of ncol columns, its
+// checkpoints every ceil(sqrt(n)) slices: columns, adjoint, checkpoints,
+// segment, partial sums; sets 0 and 1 of the context's buffers.
+struct AdjointSet {
+    DevBuf* b[5];
+    size_t bytes[5];
+};
+AdjointSet adjoint_set(bip_ctx* c, int set, int ncol, int n) {
+    const size_t state = (size_t)ncol * c->cfg.ny * c->cfg.nx * sizeof(float2);
     const int k = isqrt_up(n), nck = (n + k - 1) / k;
-    CUDA_TRY(c, ensure(set ? c->cols2 : c->cols, state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_adj[set], state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_ckpt[set], (size_t)nck * state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_seg[set], (size_t)k * state * sizeof(float2), false, s));
-    CUDA_TRY(c, ensure(c->g_gvp[set], (size_t)ncol * G * sizeof(float), false, s));
+    return AdjointSet{{set ? &c->cols2 : &c->cols, &c->g_adj[set], &c->g_ckpt[set], &c->g_seg[set], &c->g_gvp[set]},
+                      {state, state, nck * state, k * state, state / 2}};
+}
+
+bip_status adjoint_alloc(bip_ctx* c, const AdjointSet& a, cudaStream_t s) {
+    for (int i = 0; i < 5; ++i) CUDA_TRY(c, ensure(*a.b[i], a.bytes[i], false, s));
     return BIP_OK;
 }
 
-// Whether S2's adjoint sweep can have workspaces of its own beside S1's: they
-// are there already, or the device has twice their size free.
-bool adjoint_pair_fits(bip_ctx* c, int ncol, int n) {
-    const size_t G = (size_t)c->cfg.ny * c->cfg.nx, state = (size_t)ncol * G * sizeof(float2);
-    const int k = isqrt_up(n), nck = (n + k - 1) / k;
-    const size_t nv = (size_t)c->cfg.nz * G;
-    if (c->cols2.cap >= state && c->g_adj[1].cap >= state && c->g_ckpt[1].cap >= nck * state &&
-        c->g_seg[1].cap >= k * state && c->g_gvp[1].cap >= state / 2 && c->tcache.cap >= nv * sizeof(float2) &&
-        c->g_dV2.cap >= nv * sizeof(float))
-        return true;
+// Whether the two adjoint sweeps have workspaces of their own: they are there
+// already, or there is room for both sets, the transmissions and S2's
+// derivative, with as much as the second set left free beside them.  The
+// second set is held from then on, so it may take a 64th of the device at
+// most (4.4 GB: 1024^2 and 19 columns through 140 slices; sweeps of more fill
+// the chip one by one).  Nothing is allocated for a capture.
+bool adjoint_pair_fits(bip_ctx* c, const AdjointSet& s1, const AdjointSet& s2, cudaStream_t s) {
+    const size_t nv = (size_t)c->cfg.nz * c->cfg.ny * c->cfg.nx;
+    size_t grow = 0, second = 0;
+    auto count = [&](const DevBuf& b, size_t bytes) { grow += b.cap < bytes ? bytes : 0; };
+    for (int i = 0; i < 5; ++i) {
+        count(*s1.b[i], s1.bytes[i]);
+        count(*s2.b[i], s2.bytes[i]);
+        second += s2.bytes[i];
+    }
+    count(c->tcache, nv * sizeof(float2));
+    count(c->g_dV2, nv * sizeof(float));
+    if (grow == 0) return true;
+    if (capturing(s)) return false;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
-    return free_b / 2 >= (size_t)(nck + k + 3) * state + 3 * nv * sizeof(float);
+    return second <= total_b / 64 && grow + second <= free_b;
 }
 
 // dL/dV_j through the S1 sweep (psi_{j+1} = Prop(T_j psi_j)), j < the last
@@ -3444,9 +3459,9 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
     if (d_V) {
         // The two sweeps side by side (as bip_build's: their launches of a few
         // columns leave most of the chip idle), S2's derivative in a buffer of
-        // its own that is added at the end: the sums and their order are those
-        // of one sweep after the other, which a device with little memory left
-        // still runs.  Everything written is allocated before they fork.  256^2,
+        // its own that is added at the end; a device without room for both
+        // runs one after the other, without the second set an earlier call may
+        // have left.  Everything written is allocated before they fork.  256^2,
         // 40 slices, 64 sites, build to derivatives: 30.0 -> 28.8 ms (mixed), 54.1 ->
         // 53.1 (FP32).
         const size_t G = (size_t)g.ny * g.nx, nv = (size_t)g.nz * G;
@@ -3456,9 +3471,14 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
             first = std::min(first, (int)sd.plane);
         }
         const int n2 = g.nz - first;
-        const bool pair = jmax > 0 && n2 > 0 && adjoint_pair_fits(c, geo.Bp2, n2);
-        st = jmax > 0 ? adjoint_alloc(c, 0, geo.Bp1, jmax, s) : BIP_OK;
-        if (st == BIP_OK && n2 > 0) st = adjoint_alloc(c, pair ? 1 : 0, geo.Bp2, n2, s);
+        const AdjointSet set1 = adjoint_set(c, 0, geo.Bp1, std::max(jmax, 1));
+        const bool pair = jmax > 0 && n2 > 0 && adjoint_pair_fits(c, set1, adjoint_set(c, 1, geo.Bp2, n2), s);
+        if (!pair && jmax > 0 && n2 > 0 && !capturing(s) && c->g_adj[1].p) {
+            CUDA_TRY(c, cudaStreamSynchronize(s));
+            for (DevBuf* b : {&c->g_adj[1], &c->g_ckpt[1], &c->g_seg[1], &c->g_gvp[1], &c->g_dV2}) release(*b);
+        }
+        st = jmax > 0 ? adjoint_alloc(c, set1, s) : BIP_OK;
+        if (st == BIP_OK && n2 > 0) st = adjoint_alloc(c, adjoint_set(c, pair ? 1 : 0, geo.Bp2, n2), s);
         if (st != BIP_OK) return st;
         CUDA_TRY(c, cudaMemsetAsync(d_V, 0, nv * sizeof(float), s));
         if (pair) {
