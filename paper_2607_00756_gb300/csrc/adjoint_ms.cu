@@ -179,9 +179,11 @@ cudaError_t launch_adj_row(const MsPlan& p, const MsAdjArgs& a, int* groups, cud
 __global__ void gv_reduce_kernel(const float* part, int groups, int G, float* gV) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= G) return;
-    float s = gV[i];
+    // the groups first: a sweep's sum is then the same number whether it goes
+    // onto the other sweep's or into a buffer added later (gv_add_kernel)
+    float s = 0.f;
     for (int q = 0; q < groups; ++q) s += part[(size_t)q * G + i];
-    gV[i] = s;
+    gV[i] += s;
 }
 
 __global__ void gv_add_kernel(const float* __restrict__ a, size_t n, float* __restrict__ gV) {

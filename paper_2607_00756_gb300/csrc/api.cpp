@@ -3460,10 +3460,10 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
         // The two sweeps side by side (as bip_build's: their launches of a few
         // columns leave most of the chip idle), S2's derivative in a buffer of
         // its own that is added at the end; a device without room for both
-        // runs one after the other, without the second set an earlier call may
-        // have left.  Everything written is allocated before they fork.  256^2,
-        // 40 slices, 64 sites, build to derivatives: 30.0 -> 28.8 ms (mixed), 54.1 ->
-        // 53.1 (FP32).
+        // runs one after the other, to the same bits, without the second set an
+        // earlier call may have left.  Everything written is allocated before
+        // they fork.  256^2, 40 slices, 64 sites, build to derivatives: 30.0 ->
+        // 28.8 ms (mixed), 54.1 -> 53.1 (FP32).
         const size_t G = (size_t)g.ny * g.nx, nv = (size_t)g.nz * G;
         int jmax = 0, first = g.nz;
         for (auto& sd : c->sites) {

@@ -557,7 +557,7 @@ struct MsAdjArgs {
     float* gv_part;                 // [groups][ny][nx]
 };
 cudaError_t bip_ms_adj_row_pass(const MsPlan& plan, const MsAdjArgs& a, int* groups, cudaStream_t s);
-// gV[y][x] += sum_g part[g][y][x] (groups in order)
+// gV[y][x] += (sum_g part[g][y][x], groups in order)
 cudaError_t bip_gv_reduce(const float* part, int groups, int G, float* gV, cudaStream_t s);
 // gV += a, n values
 cudaError_t bip_gv_add(const float* a, size_t n, float* gV, cudaStream_t s);

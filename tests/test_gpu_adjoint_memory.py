@@ -54,3 +54,11 @@ def test_memory_for_one_set_only():
     got = run((24, 25), 4, s1 + 64 * MB)              # (S2's set: 200 MB)
     assert np.linalg.norm(got) > 0
     assert np.linalg.norm(got - want) <= 1e-6 * np.linalg.norm(want)
+
+
+def test_one_after_the_other_gives_the_bits_of_both_at_once():
+    """Sites in slices 2 and 22: both sweeps reach the slices between."""
+    want = run((2, 23, 20), 2, None)
+    state = 19 * 512 * 512 * 8
+    one = (1 + 5 + 5) * state + state // 2
+    assert np.array_equal(run((2, 23, 20), 2, one + 64 * MB), want)
