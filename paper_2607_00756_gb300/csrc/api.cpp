@@ -666,6 +666,7 @@ MsPlan plan_for(bip_ctx* c, int ncol, const DevBuf& shift) {
     p.px = (const float2*)c->px.p;
     p.shift = (const int2*)shift.p;
     p.twhw = (const float2*)c->twhw.p;
+    p.hw256 = ncol >= 128;
     return p;
 }
 
@@ -2541,6 +2542,9 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
         // the batch's exact S2 columns, exit surface to the first site plane
         MsPlan plan = plan_for(c, nd, c->shcube);
         plan.shift = (const int2*)c->shcube.p + d0;
+        // by the cube, not the chunk, so that a beam's bits do not depend on how
+        // many beams the memory takes at a time (as the k split below)
+        plan.hw256 = n_cube >= 128;
         {
             MsRowArgs a{};
             a.cols = (float2*)c->ccols.p;
@@ -2695,9 +2699,10 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
                                       Bpad, s));
                 }
             } else {
-                TIMED(c, BIP_STAGE_COUPLING, s,
-                      cgemm(c, coupling_f32(nd, (int)rowsB, K, c->xopA.p, (int64_t)perA, c->xopB.p, (int64_t)perB,
-                                            c->xm32.p, (int64_t)nch * Dpb, (int64_t)perMt, Bpad, geo.B, Dpb, nb), s));
+                CGemmF32 m = coupling_f32(nd, (int)rowsB, K, c->xopA.p, (int64_t)perA, c->xopB.p, (int64_t)perB,
+                                          c->xm32.p, (int64_t)nch * Dpb, (int64_t)perMt, Bpad, geo.B, Dpb, nb);
+                m.plan_rows = n_cube;
+                TIMED(c, BIP_STAGE_COUPLING, s, cgemm(c, m, s));
                 if (sep) {
                     CubeRasterArgs r = cra;
                     r.n_sites = nb;

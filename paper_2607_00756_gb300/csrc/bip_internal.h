@@ -115,6 +115,7 @@ struct MsPlan {
     const int2* shift;              // [ncol] propagator shift (sy, sx)
     const float2* twhw;             // nx = R1 R2 = 16 x 16, 32 x 16 or 32 x 32: exp(-2 pi i e j / nx) at
                                     // (e - 1) R1 + j, e < R2, j < R1 (the half-warp row pass); else null
+    int hw256;                      // rows of 256 points take that pass too
 };
 // row pass: [inverse row FFT] -> [T_pre] -> [stash] -> [T_post] -> [row FFT]
 struct MsRowArgs {
@@ -315,7 +316,7 @@ struct CGemmF32 {
     float2* C; int64_t scm, scn, scb;
     int ep_B, ep_n, ep_Dp;
     int tri;                        // only the column tiles that reach the diagonal or lie right of it
-    int plan_batch;                 // batch size the k split is chosen for (0: batch)
+    int plan_batch, plan_rows;      // batch size and rows the k split is chosen for (0: batch, M)
     float2* part;                   // workspace of a split k range
     int* err;
     uint64_t wait_ns;

@@ -45,6 +45,8 @@
 // written to a workspace and added in order by cgemm_sum_kernel: the result
 // does not depend on scheduling.  Every wait is bounded; on a timeout the
 // kernel sets *err, stops issuing, drains its MMAs and frees TMEM.
+#include <algorithm>
+
 #include "tc_common.cuh"
 
 namespace {
@@ -592,8 +594,8 @@ bool aligned2(const void* q, int64_t a, int64_t b, int64_t c) {
 // columns, since rows are padded to 128.  The split: the parts
 // that minimise rounds x (chunks per part + the pipeline's fill, about three
 // chunks), plus the parts' way through memory at about 2.5 KB per clock.  It
-// is chosen for plan_batch entries, so that a site's sums do not depend on
-// how full its batch is.
+// is chosen for plan_batch entries and plan_rows rows, so that a site's sums do
+// not depend on how full its batch is, nor a beam's on its cube's chunks.
 cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
     if (p.M < 1 || p.N < 1 || p.batch < 1) return cudaErrorInvalidValue;
     for (CGemmOperand* o : {&p.A, &p.B}) {
@@ -617,11 +619,12 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
     for (int mt = 0; mt < m_tiles; ++mt) p.tiles += p.n_tiles - (p.tri ? mt * 128 / p.nt : 0);
     p.steps = p.A.nper * (p.A.kper / kStep);
     const int pb = p.plan_batch > 0 ? p.plan_batch : p.batch;
-    const int64_t units = (int64_t)p.tiles * pb;
-    if (units * 16 > (1 << 26) || (int64_t)p.tiles * p.batch * 16 > (1 << 26)) return cudaErrorInvalidValue;
+    if ((int64_t)p.tiles * std::max(pb, p.batch) * 16 > (1 << 26)) return cudaErrorInvalidValue;
+    const int rows = p.plan_rows > 0 ? p.plan_rows : p.M;
+    const int64_t units = (p.plan_rows > 0 ? (int64_t)((rows + 127) / 128) * p.n_tiles : p.tiles) * pb;
     const int sms = num_sms();
     const double chunk = 2800.0;                               // clocks, whatever the width
-    const double bytes = 8.0 * pb * (double)p.M * p.cols;
+    const double bytes = 8.0 * pb * (double)rows * p.cols;
     double best = 0.0;
     p.ksplit = 1;
     for (int S = 1; S <= 16 && S * 4 <= p.steps; ++S) {

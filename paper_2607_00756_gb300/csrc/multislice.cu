@@ -647,11 +647,12 @@ cudaError_t bip_ms_row_pass(const MsPlan& p, const MsRowArgs& a, cudaStream_t s)
     switch (p.nx) {
         case 64: return launch_row<64>(p, a, s);
         case 128: return launch_row<128>(p, a, s);
-        // 256: the cube's sweeps (2048 columns: 472 -> 355 us per launch).  Parent
-        // sets stay with the radix-8 pass, 1.3% of a fit step slower: other last
-        // bits of their stashes draw the reverse pass's split-BF16 roundings anew
-        // (2.6e-5 of dL/dV).
-        case 256: return p.twhw && p.ncol >= 128 ? launch_row_hw<256>(p, a, s) : launch_row<256>(p, a, s);
+        // 256: sets of 128 columns and more, a cube's whatever its chunks (2048
+        // columns: 472 -> 355 us per launch).  Smaller parent sets stay with the
+        // radix-8 pass, 1.3% of a fit step slower: other last bits of their
+        // stashes draw the reverse pass's split-BF16 roundings anew (2.6e-5 of
+        // dL/dV).
+        case 256: return p.twhw && p.hw256 ? launch_row_hw<256>(p, a, s) : launch_row<256>(p, a, s);
         case 512: return p.twhw ? launch_row_hw<512>(p, a, s) : launch_row<512>(p, a, s);
         case 1024: return p.twhw ? launch_row_hw<1024>(p, a, s) : launch_row<1024>(p, a, s);
         case 192: return launch_row<192>(p, a, s);
