@@ -1650,6 +1650,7 @@ CubeArgs cube_args(const bip_ctx* c, const int32_t* ids, int nb, int P, float* c
     a.site_ids = ids;
     a.sites = (const SiteDev*)c->sites_d.p;
     a.n_det = c->geo.n_det;
+    a.B = c->geo.B;
     a.Bpad = c->Bpad;
     a.nch = c->nch_max;
     a.Dp = c->Dpad;

@@ -448,9 +448,9 @@ struct CubeArgs {
     int n_sites;                    // sites of this batch, added in order
     const int32_t* site_ids;
     const SiteDev* sites;
-    int n_det, Bpad, nch, Dp;       // M^(n)_{d,b} at element b m_ld + n Dp + d
+    int n_det, B, Bpad, nch, Dp;    // M^(n)_{d,b} at element b m_ld + n Dp + d
     int64_t m_ld, m_site;           // row stride, site stride
-    const float2* m32;              // the coupling, complex64
+    const float2* m32;              // the coupling, complex64 (rows past B are not read)
     const float2* C;                // [Bpad][P]
     int P;
     const double* scans;

@@ -66,13 +66,14 @@ __global__ void __launch_bounds__(kThreads) cube_kernel(CubeArgs a) {
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) ar[i][j] = ai[i][j] = 0.f;
-            for (int b0 = 0; b0 < a.Bpad; b0 += kKb) {
+            for (int b0 = 0; b0 < a.B; b0 += kKb) {
                 for (int k = threadIdx.x; k < kKb * kTile; k += kThreads) {
                     const int bb = k / kTile, x = k % kTile;
                     const int d = d0 + x, p = p0 + x;
-                    ms[bb][x] = d < a.n_det ? a.m32[(size_t)bs * a.m_site + (int64_t)(b0 + bb) * a.m_ld +
-                                                    (int64_t)n * a.Dp + d]
-                                            : make_float2(0.f, 0.f);
+                    // rows past B hold what an M of another layout left there
+                    ms[bb][x] = make_float2(0.f, 0.f);
+                    if (d < a.n_det && b0 + bb < a.B)
+                        ms[bb][x] = a.m32[(size_t)bs * a.m_site + (int64_t)(b0 + bb) * a.m_ld + (int64_t)n * a.Dp + d];
                     cs[bb][x] = p < a.P ? a.C[(size_t)(b0 + bb) * a.P + p] : make_float2(0.f, 0.f);
                 }
                 __syncthreads();
@@ -133,7 +134,7 @@ cudaError_t bip_illum(const IllumArgs& a, cudaStream_t s) {
 
 cudaError_t bip_cube_accumulate(const CubeArgs& a, cudaStream_t s) {
     if (a.n_sites < 1) return cudaSuccess;
-    if (a.Bpad % kKb || a.cube_ld < a.n_det) return cudaErrorInvalidValue;
+    if (a.Bpad % kKb || a.B > a.Bpad || a.cube_ld < a.n_det) return cudaErrorInvalidValue;
     const dim3 grid((a.n_det + kTile - 1) / kTile, (a.P + kTile - 1) / kTile);
     cube_kernel<<<grid, kThreads, 0, s>>>(a);
     return cudaGetLastError();

@@ -46,3 +46,29 @@ def test_bits_do_not_depend_on_the_chunk(env, n, prec):
     assert got[0].shape[1] == 208 and got[0].max() > 0
     for g in got[1:]:
         assert np.array_equal(g, got[0])
+
+
+@pytest.mark.parametrize("first,then", [(0, 32), (32, 0), (160, 64)])
+def test_nothing_is_left_of_a_cube_with_nan(env, first, then):
+    """A cube of transition potentials with a NaN, then one of good ones in
+    chunks of another size, on scans that are no raster: only the good one's."""
+    cfg = synth.config1().replace(cube_ky=16, cube_kx=13)
+    sp = synth.make_specimen(cfg)
+    V = torch.tensor(sp.V, dtype=torch.float32, device="cuda")
+    H = torch.tensor(sp.H, dtype=torch.complex64, device="cuda")
+    scans = sp.scans[:9] + np.random.default_rng(1).random((9, 2))
+    ctx = env(cfg, prec="fp32")
+    try:
+        ctx.build(V, sp.atoms, sp.nch)
+        per_beam = (ctx.n_sites * cfg.win ** 2 + cfg.ny * cfg.nx) * 8
+        memory = {b: b * per_beam + (b > 0) for b in (first, then)}
+        ctx.set_cube_memory(memory[then])
+        want = ctx.cube(V, H, scans).cpu().numpy()
+        bad = H.clone()
+        bad[:, 5, 7] = float("nan")
+        ctx.set_cube_memory(memory[first])
+        assert not np.isfinite(ctx.cube(V, bad, scans).cpu().numpy()).all()
+        ctx.set_cube_memory(memory[then])
+        assert np.array_equal(ctx.cube(V, H, scans).cpu().numpy(), want)
+    finally:
+        ctx.close()
