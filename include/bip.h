@@ -65,8 +65,8 @@ typedef enum {
 typedef enum {
     BIP_PREC_FP32 = 0,         /* FP32 throughout: complex64 operands, each
                                   element taken to the tensor cores as three
-                                  BF16 terms (24 bits, six products), FP32
-                                  sums; an infinite element gives NaN        */
+                                  BF16 terms (24 bits, six products; elements
+                                  below 2^-110 keep fewer), FP32 sums         */
     BIP_PREC_SPLIT_BF16 = 1,   /* tcgen05, every contraction in BF16 hi+lo
                                   (3 products per real product), FP32 acc.    */
     BIP_PREC_MIXED = 2,        /* tcgen05, coupling and Gram in BF16 (one

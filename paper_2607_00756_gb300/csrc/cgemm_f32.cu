@@ -15,8 +15,9 @@
 // the five small products first and the leading one last, so only two MMAs add
 // at full magnitude per chunk; the chunks are then added in FP32 registers with
 // round-to-nearest.  That is 16x fewer roundings per sum than a fused
-// multiply-add per k, and no long run of tensor-core additions.  An infinite
-// element gives NaN (its residual is undefined), a NaN stays one.
+// multiply-add per k, and no long run of tensor-core additions.  The whole FP32
+// range is taken, infinities and NaN as such; elements below 2^-110 (7.7e-34)
+// lose the last of their 24 bits, as BF16 ends at 2^-133.
 //
 // The complex product as one real one: an A row holds [Re (16) | Im (16)] of a
 // chunk (64 bytes), B has two rows per column n, [Re | -Im] for the real part
@@ -193,9 +194,13 @@ __device__ __forceinline__ void load8(float2 (&v)[8], const CGemmOperand& o, con
     }
 }
 
-// two FP32 values as three BF16 pairs
+// two FP32 values as three BF16 pairs.  The first two terms stay finite: past
+// the largest BF16 (3.3895e38) they are that, which leaves the rest to the
+// last term, so the largest FP32 values are exact too and an infinite one
+// comes out infinite in the last term.
 __device__ __forceinline__ uint32_t rest(float& a, float& b) {
-    const uint32_t t = pack_bf16x2(a, b);
+    uint32_t t;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(t) : "f"(b), "f"(a));
     asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\tsub.rn.f32x2 x, x, y;\n\t"
         "mov.b64 {%0, %1}, x;\n\t}"
         : "+f"(a), "+f"(b)
