@@ -621,7 +621,7 @@ cudaError_t bip_cgemm_plan(CGemmF32& p, size_t* part_elems) {
     p.n_tiles = (p.cols + p.nt - 1) / p.nt;
     const int m_tiles = (p.M + 127) / 128;
     p.tiles = 0;
-    for (int mt = 0; mt < m_tiles; ++mt) p.tiles += p.n_tiles - (p.tri ? mt * 128 / p.nt : 0);
+    for (int mt = 0; mt < m_tiles; ++mt) p.tiles += std::max(0, p.n_tiles - (p.tri ? mt * 128 / p.nt : 0));
     p.steps = p.A.nper * (p.A.kper / kStep);
     const int pb = p.plan_batch > 0 ? p.plan_batch : p.batch;
     if ((int64_t)p.tiles * std::max(pb, p.batch) * 16 > (1 << 26)) return cudaErrorInvalidValue;

@@ -1,5 +1,6 @@
 """The FP32 complex contraction (bip_debug_cgemm) at the ends of the FP32
-range: the largest finite elements and infinite ones."""
+range, the largest finite elements and infinite ones, and the triangle of a
+product that is not square."""
 import pytest
 
 import synth
@@ -85,3 +86,17 @@ def test_infinite_elements(env, layout, side):
         assert torch.isinf(want).sum() == 2 * (N if side == 0 else M)
         assert torch.equal(torch.isinf(got), torch.isinf(want)) and not torch.isnan(got).any()
         assert torch.equal(got[torch.isinf(want)], want[torch.isinf(want)])
+
+
+@pytest.mark.parametrize("M,N", [(512, 256), (300, 129), (1000, 40), (129, 500)])
+def test_upper_triangle_of_a_rectangle(env, M, N):
+    """Flag 4 with more rows than columns, and with fewer: every entry on or
+    above the diagonal is written."""
+    capi, ctx = env
+    K = 48
+    (A, sA), (B, sB) = operands("kk", M, N, K)
+    C = torch.full((M, N), float("nan"), dtype=torch.complex64, device="cuda")
+    capi.bip_debug_cgemm(ctx, M, N, K, 1, 1, A, sA, B, sB, 4, None, C)
+    a, b = A.to(torch.complex128), B.to(torch.complex128)
+    up = torch.ones(M, N, dtype=torch.bool, device="cuda").triu()
+    assert torch.all((C - a @ b.T).abs()[up] <= ((K / 16 + 40) * 2.0 ** -24 * (a.abs() @ b.abs().T))[up])
