@@ -2866,7 +2866,7 @@ bip_status bip_debug_cgemm(bip_ctx* c, int32_t M, int32_t N, int32_t K, int32_t 
 bip_status bip_debug_split(bip_ctx* c, int32_t rows, int32_t cols, const void* src, int64_t s_row, int64_t s_col,
                            int32_t d_cols, int32_t dcol0, int32_t conj, void* dst, void* stream) {
     if (!c || !src || !dst) return BIP_ERR_INVALID_ARG;
-    if (rows < 1 || cols < 1 || dcol0 < 0 || dcol0 + cols > d_cols || (s_row != 1 && s_col != 1))
+    if (rows < 1 || cols < 1 || dcol0 < 0 || (int64_t)dcol0 + cols > d_cols || (s_row != 1 && s_col != 1))
         return fail(c, BIP_ERR_INVALID_ARG, "bad size or stride");
     SplitArgs a{(const float2*)src, s_row, s_col, 0, rows, cols, 1, (uint16_t*)dst, 0, rows, d_cols, dcol0, conj};
     CUDA_TRY(c, bip_split_planes(a, (cudaStream_t)stream));

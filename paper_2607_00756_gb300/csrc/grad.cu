@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256) split_planes_kernel(SplitArgs a, bool src
 }  // namespace
 
 cudaError_t bip_split_planes(const SplitArgs& a, cudaStream_t s) {
-    if (a.rows < 1 || a.cols < 1 || a.batch < 1 || a.rows > a.d_rows || a.dcol0 + a.cols > a.d_cols)
+    if (a.rows < 1 || a.cols < 1 || a.batch < 1 || a.rows > a.d_rows || (int64_t)a.dcol0 + a.cols > a.d_cols)
         return cudaErrorInvalidValue;
     if (a.s_col != 1 && a.s_row != 1) return cudaErrorInvalidValue;
     const dim3 grid((a.cols + 63) / 64, (a.rows + 31) / 32, a.batch);
