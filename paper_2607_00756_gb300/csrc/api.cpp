@@ -266,6 +266,8 @@ bool capturing(cudaStream_t s) {
     return st != cudaStreamCaptureStatusNone;
 }
 
+// Host to device from pageable memory, which the copy has left when it returns
+// (page-locked memory is read whenever the stream gets there).
 template <class T>
 cudaError_t upload(DevBuf& b, const std::vector<T>& h, cudaStream_t s) {
     cudaError_t e = ensure(b, h.size() * sizeof(T), false, s);
@@ -1745,10 +1747,12 @@ bip_status run_map(bip_ctx* c, const void* H, const double* scans, int32_t P, fl
         if (capturing(s))
             return fail(c, BIP_ERR_INVALID_ARG,
                         "a captured map must repeat the scans of the capture-safe warm-up call");
-        CUDA_TRY(c, ensure(c->scans_d, (size_t)P * 2 * sizeof(double), false, s));
-        CUDA_TRY(c, cudaMemcpyAsync(c->scans_d.p, scans, (size_t)P * 2 * sizeof(double), cudaMemcpyHostToDevice, s));
-        c->scans_cache.assign(scans, scans + 2 * P);
+        // (from the context's copy: the caller's list may be page-locked)
         c->ray_scans = false;
+        c->scans_cache.clear();
+        std::vector<double> list(scans, scans + 2 * (size_t)P);
+        CUDA_TRY(c, upload(c->scans_d, list, s));
+        c->scans_cache.swap(list);
     }
     float* partial = partial_out;
     // beam order: the map as |M c|^2 summed over the detector beams on the
@@ -2437,9 +2441,8 @@ bip_status run_cube_exact(bip_ctx* c, const float* V, const void* H, const doubl
     const size_t G = (size_t)g.ny * g.nx;
     const int n_cube = geo.n_cube;
 
-    CUDA_TRY(c, ensure(c->scans_d, (size_t)P * 2 * sizeof(double), false, s));
-    CUDA_TRY(c, cudaMemcpyAsync(c->scans_d.p, scans, (size_t)P * 2 * sizeof(double), cudaMemcpyHostToDevice, s));
     c->scans_cache.clear();
+    CUDA_TRY(c, upload(c->scans_d, std::vector<double>(scans, scans + 2 * (size_t)P), s));
     CUDA_TRY(c, ensure(c->illum, (size_t)Bpad * P * sizeof(float2), false, s));
     IllumArgs ia{P, geo.B, Bpad, (const int2*)c->hbeam.p, (const double2*)c->coef.p, (const double*)c->scans_d.p,
                  g.ny, g.nx, (float2*)c->illum.p};
@@ -3137,11 +3140,11 @@ bip_status bip_set_aberrations(bip_ctx* c, double defocus, double cs, void* stre
 
 // The context's own copy of a scan list for a graph to copy from at every
 // replay, when the caller's may be gone; one copy per list, until bip_destroy.
-static const double* kept_scans(bip_ctx* c, const double* scans, int P) {
+static const std::vector<double>& kept_scans(bip_ctx* c, const double* scans, int P) {
     for (const auto& v : c->captured_scans)
-        if (v.size() == (size_t)P * 2 && std::equal(v.begin(), v.end(), scans)) return v.data();
+        if (v.size() == (size_t)P * 2 && std::equal(v.begin(), v.end(), scans)) return v;
     c->captured_scans.emplace_back(scans, scans + 2 * (size_t)P);
-    return c->captured_scans.back().data();
+    return c->captured_scans.back();
 }
 
 static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const double* scan_px, int32_t P,
@@ -3180,9 +3183,11 @@ static bip_status coreloss_grad(bip_ctx* c, const float* V, const void* H, const
     }
     // FP32 contraction per batch of sites: S2, H_n S1 and S1 windows, M (as
     // Mt[b][(n, d)]), Q, then the reverse steps
-    CUDA_TRY(c, ensure(c->g_scans, (size_t)P * 2 * sizeof(double), false, s));
-    CUDA_TRY(c, cudaMemcpyAsync(c->g_scans.p, capturing(s) ? kept_scans(c, scan_px, P) : scan_px,
-                                (size_t)P * 2 * sizeof(double), cudaMemcpyHostToDevice, s));
+    std::vector<double> list;
+    const std::vector<double>* src = &list;
+    if (capturing(s)) src = &kept_scans(c, scan_px, P);
+    else list.assign(scan_px, scan_px + 2 * (size_t)P);
+    CUDA_TRY(c, upload(c->g_scans, *src, s));
     CUDA_TRY(c, ensure(c->illum, (size_t)Bpad * P * sizeof(float2), false, s));
     IllumArgs ia{P, B, Bpad, (const int2*)c->hbeam.p, (const double2*)c->coef.p, (const double*)c->g_scans.p, g.ny,
                  g.nx, (float2*)c->illum.p};

@@ -77,3 +77,27 @@ def test_captured_gradient_keeps_its_scans(env):
         capi.bip_check_errors(ctx.ctx)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("name", ["map", "sites", "grad", "cube"])
+def test_host_list_may_change_when_the_call_returns(env, name):
+    """A scan list in page-locked memory, from which the device copies at its
+    own time, overwritten as soon as an FP32 call behind other work has
+    returned."""
+    capi, make, sp, other, H, g = env
+    V = torch.tensor(sp.V, dtype=torch.float32, device="cuda")
+    ctx = make("fp32")
+    call = {"map": lambda s: ctx.map(H, s), "sites": lambda s: ctx.sites(H, s), "cube": lambda s: ctx.cube(V, H, s),
+            "grad": lambda s: torch.view_as_real(ctx.grad(H, s, g, occ=False, aberr=False)["H"])}[name]
+    try:
+        want = call(sp.scans)
+        pinned = torch.tensor(sp.scans).pin_memory()
+        torch.cuda.synchronize()
+        torch.cuda._sleep(400_000_000)
+        got = call(pinned.numpy())
+        pinned.copy_(torch.tensor(other))
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
+        capi.bip_check_errors(ctx.ctx)
+    finally:
+        ctx.close()
