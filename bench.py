@@ -824,13 +824,13 @@ def stage_roofline(cfg, path, stage, ms, n, steps, info, geo_sizes):
     if stage in ("coupling", "gram", "quadform"):
         # per launch: the step's work over the step's launches of this stage
         per_launch = alg[stage] / (n / steps)
-        if stage == "quadform" or path == "fp32":
+        if stage == "quadform":
             achieved = per_launch / (ms_launch / 1e3) / 1e12
             out.update(bound="alu", achieved=achieved, peak=fp32_peak, unit="TFLOP/s", peak_source=fp32_src)
         else:
             # the method's own flops (one complex product = 8 flop): the
-            # split-BF16 path's three BF16 products per real product are
-            # its cost, not work, and are not counted
+            # split-BF16 path's three BF16 products per real product and the
+            # FP32 path's six are their cost, not work, and are not counted
             achieved = per_launch / (ms_launch / 1e3) / 1e12
             peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
             src = f"{info['peak_kind']} bf16 sustained"

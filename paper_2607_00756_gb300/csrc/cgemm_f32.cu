@@ -35,7 +35,7 @@
 //   warp 16      TMEM allocator and MMA issuer (40; warps 17-19 idle).
 // What bounds it: the cutting warps (latency: the loads of a chunk, then about
 // 500 dependent instructions per warp), 2800 clocks per chunk of a 128 x 128
-// tile where its MMAs take 12 x 128.  Measured on 19 x 1024 x 1024 x 4096:
+// tile where its twelve MMAs take about 1900.  Measured on 19 x 1024 x 1024 x 4096:
 // 220 TFLOP/s of complex products (SIMT FFMA, 64 x 64 tiles: 47); two groups
 // of four cutting warps taking chunks in turn 209-218, sixteen cutting warps
 // of 40 registers 160, loads issued between the cutting of A and of B 219, two
